@@ -199,7 +199,6 @@ def algorithmic(wl, stats, proc_inst, evals=0):
     N = A * K
     GV = V * N
     P = stats["n_pixels"]
-    I = stats["n_instances"]
     anc_b = 12 + 4 * 32 + 12 * K + 12          # pos, feat, offsets, scaling
     rec3d = 64 + 4 * NF                         # mean|o, scale, quat, colour, features
     n_out = K * (11 + NF)
@@ -212,12 +211,11 @@ def algorithmic(wl, stats, proc_inst, evals=0):
     passes = lambda bits: (bits + 7) // 8
     return {
         "decode_fwd": dict(bytes=A * anc_b + GV * rec3d, flops=A * V * row_fwd),
-        "project": dict(bytes=GV * (48 + 56)),
+        "project": dict(bytes=GV * (48 + 68)),
         "depth_sort": dict(bytes=passes(32 + (math.ceil(math.log2(V)) if V > 1 else 0)) * GV * 32),
-        "offsets": dict(bytes=GV * (4 + 4 + 4 + 8)),
-        "emit": dict(bytes=GV * 24 + I * 8),
-        "tile_sort": dict(bytes=passes(stats["key_bits"]) * I * 20),
-        "ranges": dict(bytes=I * 8 + stats["n_tiles"] * 8),
+        # a packed span a Gaussian-view, a word a list entry and tile
+        "tile_count": dict(bytes=GV * 20),
+        "tile_lists": dict(bytes=GV * 20 + stats["n_listed"] * 4 + stats["n_tiles"] * 8),
         "composite_fwd": dict(bytes=proc_inst * inst_b + P * pix_out, flops=evals * (2 * (NF + 4) + 12)),
         "loss": dict(bytes=P * 4 * (3 * (3 + 1 + NF) + 1)),
         # gradient records: at most one per read instance receives an atomic add

@@ -75,8 +75,8 @@ typedef struct {
                          with the t_min reading), so a cap changes nothing unless a
                          pixel is still open at the end of a cut list: the forward
                          then sorts that batch again without the cap and blends it
-                         again (ups_stats.list_refills).  Views of more than 16383
-                         tiles in total are never capped. */
+                         again (ups_stats.list_refills).  Batches with a view of
+                         more than 8191 tiles are never capped. */
     int opacity_tanh; /* 1: decoded opacity o = tanh(y) (the Scaffold-GS decode the
                          paper cites for Eq. 8-9) instead of sigmoid(y); the
                          projection's cull of o < alpha_min then drops every

@@ -112,21 +112,26 @@ cudaError_t radix_sort_u32(uint32_t **key_io, uint32_t **key_alt, uint32_t **val
 cudaError_t radix_sort_u64(uint64_t **key_io, uint64_t **key_alt, uint32_t **val_io,
                            uint32_t **val_alt, size_t n, int end_bit, SortScratch &s,
                            cudaStream_t st);
-// One-pass stable sort of (key, value) pairs by keys < nbins <= kMaxBucketBins
-// (tile ids).  Bucket d keeps its first min(count_d, cap) values (cap =
-// kNoListCap: all; a finite cap needs cap <= kMaxListCap and nbins <
-// kMaxBucketBins), written in key order to vals_out; ranges[d] is the kept
-// [start, end) and bit d of trunc[(nbins + 31) / 32] is set when bucket d
-// lost values to the cap.  scratch: bucket_sort_scratch_bytes.  gate (no
-// cap only): when non-null the kernels do nothing unless *gate != 0.
-constexpr int kMaxBucketBins = 1 << 14;
+// Tile lists of the depth-ordered Gaussian-views (bin.cu): tile t of all
+// views keeps the first min(count, cap) Gaussian-views that meet it (cap =
+// kNoListCap: all), in depth order, at lists[ranges[t].x .. ranges[t].y); bit
+// t of trunc is set when it lost some.  Views of at most kMaxBinTiles tiles.
+// bin_count fills scratch (bin_scratch_bytes); bin_lists may follow it more
+// than once.  n: entries lists has room for (>= the tile instances if cap =
+// kNoListCap); gate: when non-null its kernels do nothing unless *gate != 0.
+constexpr int kMaxBinTiles = 8191;
 constexpr int kMaxListCap = 32767;
 constexpr uint32_t kNoListCap = 0xffffffffu;
-size_t bucket_sort_scratch_bytes(size_t n, int nbins, int num_sms);
-cudaError_t bucket_sort_u32(const uint32_t *keys, const uint32_t *vals, uint32_t *vals_out, size_t n, int nbins,
-                            uint32_t cap, uint2 *ranges, uint32_t *trunc, void *scratch, size_t scratch_bytes,
-                            int num_sms, cudaStream_t st, const int *gate = nullptr);
-// keys[i] = t for every i in ranges[t] (the sorted keys of a bucket sort)
+bool bin_supported(const ViewTable &vt);
+size_t bin_scratch_bytes(const ViewTable &vt, int N, int num_sms);
+cudaError_t bin_count(const ViewTable &vt, float alpha_min, int N, const uint32_t *sorted_gv, const uint4 *span,
+                      const uint4 *more, const float4 *xyzo, const float4 *conic, void *scratch, int num_sms, cudaStream_t st);
+cudaError_t bin_lists(const ViewTable &vt, float alpha_min, int N, const uint32_t *sorted_gv, const uint4 *span,
+                      const uint4 *more, const float4 *xyzo, const float4 *conic, void *scratch, uint32_t cap, uint32_t n, uint2 *ranges,
+                      uint32_t *trunc, uint32_t *lists, int num_sms, cudaStream_t st, const int *gate = nullptr);
+// the projection spreads its sum of tile instances over this many counters
+constexpr int kInstCounters = 32;
+// keys[i] = t for every i in ranges[t] (the tile of every list entry)
 cudaError_t keys_from_ranges(const uint2 *ranges, int nbins, uint32_t *keys, cudaStream_t st);
 // C (column-major m x n, leading dimension ldc) = alpha op(A) op(B) + beta C
 // in FP32 on the CUDA cores (op = transpose when ta / tb); column-major A

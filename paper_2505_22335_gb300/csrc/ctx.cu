@@ -2,6 +2,7 @@
 // and the order of kernel launches for decode, forward, loss and backward.
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -10,18 +11,17 @@
 
 #include "common.cuh"
 #include "decode_bwd.cuh"
+#include "tiles.cuh"
 
 namespace ups {
 
 // launchers implemented in the other translation units
-cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                           int total, const ups_gaussians &g, float4 *xyzo, float4 *conic,
-                           uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
-                           cudaStream_t st);
-cudaError_t launch_project_k32(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                               int total, const ups_gaussians &g, float4 *xyzo, float4 *conic,
-                               uint2 *rect, uint32_t *count, uint32_t *dkey32, uint32_t *dval,
-                               int vbits, cudaStream_t st);
+cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
+                           float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
+                           uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
+cudaError_t launch_project_k32(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
+                               float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint32_t *dkey32,
+                               uint32_t *dval, int vbits, uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
 cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *count, uint32_t *out,
                                  int total, cudaStream_t st);
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
@@ -129,16 +129,22 @@ struct ups_ctx {
     ups_images img{};
     bool have_bwd = false;
     // scratch
-    DevBuf xyzo, conic, rect, count, dkey0, dkey1, dval0, dval1, cnt_sorted, off, scan_scr;
-    DevBuf ikey0, ikey1, ival0, ival1, ranges, g2;
+    DevBuf xyzo, conic, rect, count, span, more, dkey0, dkey1, dval0, dval1, bin_scr, lists, ranges, g2;
+    // views too large for the row-wise tile lists: instances, their offsets and sort buffers
+    DevBuf cnt_sorted, off, scan_scr, ikey0, ikey1, ival0, ival1;
     DevBuf dec_scratch;  // decode backward: X, H, dL/dY, dL/dZ rows for the weight gradients
     SortScratch sort;
     uint32_t *dval_sorted = nullptr, *ikey_sorted = nullptr, *ival_sorted = nullptr;
-    // pinned: [0] instance count, [1] device error / list-cap flag, [2] the
-    // last tile range
-    uint64_t *h_total = nullptr;
-    int *d_err = nullptr;         // set by kernels whose bounded waits ran out
-    int *d_trunc_flag = nullptr;  // set by the forward blend: a capped list was too short
+    // device words of a forward and their pinned copy: the instance counters
+    // and the list flag (cleared by every forward), the error flag
+    struct Words {
+        unsigned long long n_inst[kInstCounters];
+        int trunc_flag;  // set by the forward blend: a capped list was too short
+        int err;         // set by kernels whose bounded waits ran out
+    };
+    Words *d_words = nullptr, *h_words = nullptr;
+    cudaEvent_t words_ready = nullptr;  // the pinned copy has arrived
+    int *d_err = nullptr, *d_trunc_flag = nullptr;  // into d_words
     DevBuf trunc;                 // per-tile bit: the list cap cut the tile's list
     bool capped = false;          // the last forward capped its tile lists
     DevBuf lift_scr;              // feature-lifting scratch of one view
@@ -288,6 +294,39 @@ ups_status set_device(ups_ctx *c) {
     return UPS_OK;
 }
 
+// Tile lists of views too large for the row-wise kernels: every (tile,
+// Gaussian) instance of the depth-ordered Gaussian-views dv is written, then
+// sorted by tile (stable: depth order is kept inside each tile).
+ups_status instance_lists(ups_ctx *c, const uint32_t *dv, size_t total, cudaStream_t st) {
+    const ViewTable &vt = c->vt;
+    const size_t n_inst = c->n_inst, bytes = std::max<size_t>(n_inst, 1) * sizeof(uint32_t);
+    UPS_CUDA(c, c->cnt_sorted.reserve(total * sizeof(uint32_t)));
+    UPS_CUDA(c, c->off.reserve((total + 1) * sizeof(uint64_t)));
+    UPS_CUDA(c, c->scan_scr.reserve(scan_scratch_bytes(total)));
+    for (DevBuf *b : {&c->ikey0, &c->ikey1, &c->ival0, &c->ival1}) UPS_CUDA(c, b->reserve(bytes));
+    stage_begin(c, "offsets", st);
+    UPS_CUDA(c, launch_gather_counts(dv, c->count.as<uint32_t>(), c->cnt_sorted.as<uint32_t>(), (int)total, st));
+    UPS_CUDA(c, exclusive_scan_u32_u64(c->cnt_sorted.as<uint32_t>(), c->off.as<uint64_t>(), total,
+                                       c->scan_scr.ptr, st));
+    stage_end(c, st, 4);
+    uint32_t *ik = c->ikey0.as<uint32_t>(), *ik_alt = c->ikey1.as<uint32_t>();
+    uint32_t *iv = c->ival0.as<uint32_t>(), *iv_alt = c->ival1.as<uint32_t>();
+    stage_begin(c, "emit", st);
+    UPS_CUDA(c, launch_emit(vt, c->bp, c->N, (int)total, dv, c->off.as<uint64_t>(), c->rect.as<uint2>(),
+                            c->xyzo.as<float4>(), c->conic.as<float4>(), ik, iv, st));
+    stage_end(c, st, 1);
+    stage_begin(c, "tile_sort", st);
+    UPS_CUDA(c, radix_sort_u32(&ik, &ik_alt, &iv, &iv_alt, n_inst, c->key_bits, c->sort, st));
+    stage_end(c, st, radix_kernels(n_inst, c->key_bits));
+    c->ikey_sorted = ik;
+    c->ival_sorted = iv;
+    stage_begin(c, "ranges", st);
+    UPS_CUDA(c, cudaMemsetAsync(c->ranges.ptr, 0, (size_t)vt.total_tiles * sizeof(uint2), st));
+    UPS_CUDA(c, launch_ranges(ik, (uint32_t)n_inst, c->ranges.as<uint2>(), st));
+    stage_end(c, st, n_inst ? 1 : 0);
+    return UPS_OK;
+}
+
 }  // namespace
 
 namespace ups {
@@ -407,16 +446,17 @@ ups_status ups_create(const ups_config *cfg, int device, ups_ctx **out) {
     ctx->device = device;
     e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
-    if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_total, 4 * sizeof(uint64_t));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(ctx->d_err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_trunc_flag, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(ctx->d_trunc_flag, 0, sizeof(int));
+    if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_words, sizeof(ups_ctx::Words));
+    if (e == cudaSuccess) e = cudaMalloc(&ctx->d_words, sizeof(ups_ctx::Words));
+    if (e == cudaSuccess) e = cudaMemset(ctx->d_words, 0, sizeof(ups_ctx::Words));
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->words_ready, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         g_create_error = std::string("ups_create: ") + cudaGetErrorString(e);
-        delete ctx;
+        ups_destroy(ctx);
         return UPS_ERR_CUDA;
     }
+    ctx->d_err = &ctx->d_words->err;
+    ctx->d_trunc_flag = &ctx->d_words->trunc_flag;
     ctx->bp = BlendParams{c.alpha_min, c.alpha_max, c.t_min, c.dilation, c.near_z};
     *out = ctx;
     return UPS_OK;
@@ -425,14 +465,14 @@ ups_status ups_create(const ups_config *cfg, int device, ups_ctx **out) {
 ups_status ups_destroy(ups_ctx *c) {
     if (!c) return UPS_OK;
     cudaSetDevice(c->device);
-    DevBuf *bufs[] = {&c->xyzo, &c->conic, &c->rect, &c->count, &c->dkey0, &c->dkey1, &c->dval0,
-                      &c->dval1, &c->cnt_sorted, &c->off, &c->scan_scr, &c->ikey0, &c->ikey1,
+    DevBuf *bufs[] = {&c->xyzo, &c->conic, &c->rect, &c->count, &c->span, &c->more, &c->bin_scr, &c->lists, &c->dkey0,
+                      &c->dkey1, &c->dval0, &c->dval1, &c->cnt_sorted, &c->off, &c->scan_scr, &c->ikey0, &c->ikey1,
                       &c->ival0, &c->ival1, &c->ranges, &c->g2, &c->dec_scratch, &c->sort.hist, &c->trunc, &c->lift_scr, &c->ssim_g, &c->unc_scr, &c->anchor_scr};
     for (DevBuf *b : bufs) b->release();
-    if (c->h_total) cudaFreeHost(c->h_total);
+    if (c->h_words) cudaFreeHost(c->h_words);
     if (c->h_anchor) cudaFreeHost(c->h_anchor);
-    if (c->d_err) cudaFree(c->d_err);
-    if (c->d_trunc_flag) cudaFree(c->d_trunc_flag);
+    if (c->d_words) cudaFree(c->d_words);
+    if (c->words_ready) cudaEventDestroy(c->words_ready);
     for (auto &r : c->pending) {
         cudaEventDestroy(r.a);
         cudaEventDestroy(r.b);
@@ -544,10 +584,17 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     UPS_CUDA(c, c->dkey1.reserve(total * sizeof(uint64_t)));
     UPS_CUDA(c, c->dval0.reserve(total * sizeof(uint32_t)));
     UPS_CUDA(c, c->dval1.reserve(total * sizeof(uint32_t)));
-    UPS_CUDA(c, c->cnt_sorted.reserve(total * sizeof(uint32_t)));
-    UPS_CUDA(c, c->off.reserve((total + 1) * sizeof(uint64_t)));
-    UPS_CUDA(c, c->scan_scr.reserve(scan_scratch_bytes(total)));
     UPS_CUDA(c, c->ranges.reserve((size_t)vt.total_tiles * sizeof(uint2)));
+    // tile lists straight from the depth order, unless a view has more tiles
+    // than the row-wise kernels take
+    const bool rowwise = bin_supported(vt);
+    if (rowwise) {
+        UPS_CUDA(c, c->span.reserve(total * sizeof(uint4)));
+        UPS_CUDA(c, c->more.reserve(total * kSpanMore * sizeof(uint4)));
+        UPS_CUDA(c, c->bin_scr.reserve(bin_scratch_bytes(vt, c->N, c->num_sms)));
+        UPS_CUDA(c, c->trunc.reserve(((size_t)vt.total_tiles + 31) / 32 * 4));
+    }
+    uint4 *span = rowwise ? c->span.as<uint4>() : nullptr, *more = rowwise ? c->more.as<uint4>() : nullptr;
 
     // (view, depth) order of the Gaussian-views: 32-bit keys (view in the top
     // bits, depth bits above 0.125 m below) when the view index fits in 4 bits
@@ -555,16 +602,21 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     int vbits = bits_for((size_t)n_views);
     const bool k32 = vbits <= 4 && c->bp.near_z >= 0.125f;
     uint32_t *dv = c->dval0.as<uint32_t>(), *dv_alt = c->dval1.as<uint32_t>();
+    UPS_CUDA(c, cudaMemsetAsync(c->d_words, 0, offsetof(ups_ctx::Words, err), st));
     stage_begin(c, "project", st);
     if (k32)
-        UPS_CUDA(c, launch_project_k32(vt, c->bp, c->N, c->per_view, (int)total, *g, c->xyzo.as<float4>(),
-                                       c->conic.as<float4>(), c->rect.as<uint2>(), c->count.as<uint32_t>(),
-                                       c->dkey0.as<uint32_t>(), dv, vbits, st));
+        UPS_CUDA(c, launch_project_k32(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
+                                       c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint32_t>(), dv, vbits,
+                                       span, more, c->d_words->n_inst, st));
     else
-        UPS_CUDA(c, launch_project(vt, c->bp, c->N, c->per_view, (int)total, *g, c->xyzo.as<float4>(),
-                                   c->conic.as<float4>(), c->rect.as<uint2>(), c->count.as<uint32_t>(),
-                                   c->dkey0.as<uint64_t>(), dv, st));
+        UPS_CUDA(c, launch_project(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
+                                   c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint64_t>(), dv, span, more,
+                                   c->d_words->n_inst, st));
     stage_end(c, st, 1);
+    // the host needs the instance count to size the lists: its copy follows the
+    // projection, so that the GPU sorts and counts while the host waits for it
+    UPS_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_words, sizeof(ups_ctx::Words), cudaMemcpyDeviceToHost, st));
+    UPS_CUDA(c, cudaEventRecord(c->words_ready, st));
     stage_begin(c, "depth_sort", st);
     if (k32) {
         uint32_t *dk = c->dkey0.as<uint32_t>(), *dk_alt = c->dkey1.as<uint32_t>();
@@ -576,64 +628,44 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
         stage_end(c, st, radix_kernels(total, 32 + vbits));
     }
     c->dval_sorted = dv;
-    stage_begin(c, "offsets", st);
-    UPS_CUDA(c, launch_gather_counts(dv, c->count.as<uint32_t>(), c->cnt_sorted.as<uint32_t>(), (int)total, st));
-    UPS_CUDA(c, exclusive_scan_u32_u64(c->cnt_sorted.as<uint32_t>(), c->off.as<uint64_t>(), total,
-                                       c->scan_scr.ptr, st));
-    stage_end(c, st, 4);
-    UPS_CUDA(c, cudaMemcpyAsync(c->h_total, c->off.as<uint64_t>() + total, sizeof(uint64_t),
-                                cudaMemcpyDeviceToHost, st));
-    c->h_total[1] = 0;
-    UPS_CUDA(c, cudaMemcpyAsync(c->h_total + 1, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, st));
-    UPS_CUDA(c, cudaStreamSynchronize(st));
-    if (c->h_total[1] != 0) {
+    if (rowwise) {
+        stage_begin(c, "tile_count", st);
+        UPS_CUDA(c, bin_count(vt, c->bp.alpha_min, c->N, dv, span, more, c->xyzo.as<float4>(), c->conic.as<float4>(),
+                              c->bin_scr.ptr, c->num_sms, st));
+        stage_end(c, st, 2);
+    }
+    UPS_CUDA(c, cudaEventSynchronize(c->words_ready));
+    if (c->h_words->err != 0) {
         cudaMemsetAsync(c->d_err, 0, sizeof(int), st);
         return fail(c, UPS_ERR_TIMEOUT, "a bounded wait of a kernel ran out of polls in an earlier launch");
     }
-    const uint64_t n_inst = *c->h_total;
+    uint64_t n_inst = 0;
+    for (int i = 0; i < kInstCounters; ++i) n_inst += c->h_words->n_inst[i];
     if (n_inst >= (uint64_t)UINT32_MAX) return fail(c, UPS_ERR_CAPACITY, "more than 2^32 tile instances");
     c->n_inst = (size_t)n_inst;
-    UPS_CUDA(c, c->ikey0.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
-    UPS_CUDA(c, c->ikey1.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
-    UPS_CUDA(c, c->ival0.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
-    UPS_CUDA(c, c->ival1.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
-    uint32_t *ik = c->ikey0.as<uint32_t>(), *ik_alt = c->ikey1.as<uint32_t>();
-    uint32_t *iv = c->ival0.as<uint32_t>(), *iv_alt = c->ival1.as<uint32_t>();
-    stage_begin(c, "emit", st);
-    UPS_CUDA(c, launch_emit(vt, c->bp, c->N, (int)total, dv, c->off.as<uint64_t>(), c->rect.as<uint2>(),
-                            c->xyzo.as<float4>(), c->conic.as<float4>(), ik, iv, st));
-    stage_end(c, st, 1);
-    // stable bucket by (view, tile): depth order is kept inside each tile
     c->key_bits = bits_for((size_t)vt.total_tiles);
-    stage_begin(c, "tile_sort", st);
-    const uint32_t cap = c->cfg.list_cap < 0 || vt.total_tiles >= kMaxBucketBins
+    const uint32_t cap = !rowwise || c->cfg.list_cap < 0
                              ? kNoListCap
                              : (uint32_t)(c->cfg.list_cap == 0 ? 1024 : c->cfg.list_cap);
-    const bool bucket = vt.total_tiles <= kMaxBucketBins;
-    if (bucket) {
-        // one pass: values in tile order and the tile ranges; the sorted keys
-        // are only rebuilt (from the ranges) when inspected
-        const size_t need = bucket_sort_scratch_bytes(n_inst, vt.total_tiles, c->num_sms);
-        UPS_CUDA(c, c->sort.hist.reserve(std::max<size_t>(need, 256)));
-        UPS_CUDA(c, c->trunc.reserve(((size_t)vt.total_tiles + 31) / 32 * 4));
-        UPS_CUDA(c, bucket_sort_u32(ik, iv, iv_alt, n_inst, vt.total_tiles, cap, c->ranges.as<uint2>(),
-                                    c->trunc.as<uint32_t>(), c->sort.hist.ptr, c->sort.hist.bytes, c->num_sms, st));
-        stage_end(c, st, n_inst ? 6 : 0);
-        c->ikey_sorted = nullptr;
-        c->ival_sorted = iv_alt;
+    c->ikey_sorted = nullptr;  // rebuilt from the ranges when inspected
+    auto lists = [&](uint32_t keep, const int *gate) {
+        return bin_lists(vt, c->bp.alpha_min, c->N, dv, span, more, c->xyzo.as<float4>(), c->conic.as<float4>(),
+                         c->bin_scr.ptr, keep, (uint32_t)n_inst, c->ranges.as<uint2>(), c->trunc.as<uint32_t>(),
+                         c->lists.as<uint32_t>(), c->num_sms, st, gate);
+    };
+    if (rowwise) {
+        // room for every instance: a capped list may have to be rebuilt whole
+        UPS_CUDA(c, c->lists.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
+        stage_begin(c, "tile_lists", st);
+        UPS_CUDA(c, lists(cap, nullptr));
+        stage_end(c, st, n_inst ? 2 : 1);
+        c->ival_sorted = c->lists.as<uint32_t>();
     } else {
-        UPS_CUDA(c, radix_sort_u32(&ik, &ik_alt, &iv, &iv_alt, n_inst, c->key_bits, c->sort, st));
-        stage_end(c, st, radix_kernels(n_inst, c->key_bits));
-        c->ikey_sorted = ik;
-        c->ival_sorted = iv;
-        stage_begin(c, "ranges", st);
-        UPS_CUDA(c, cudaMemsetAsync(c->ranges.ptr, 0, (size_t)vt.total_tiles * sizeof(uint2), st));
-        UPS_CUDA(c, launch_ranges(ik, (uint32_t)n_inst, c->ranges.as<uint2>(), st));
-        stage_end(c, st, n_inst ? 1 : 0);
+        ups_status ls = instance_lists(c, dv, total, st);
+        if (ls != UPS_OK) return ls;
     }
-    const bool capped = bucket && cap != kNoListCap && n_inst > 0;
+    const bool capped = cap != kNoListCap && n_inst > 0;
     c->capped = capped;
-    if (capped) UPS_CUDA(c, cudaMemsetAsync(c->d_trunc_flag, 0, sizeof(int), st));
     stage_begin(c, "composite_fwd", st);
     UPS_CUDA(c, launch_composite_fwd(vt, c->bp, c->cfg.n_feat, c->N, c->per_view, c->ranges.as<uint2>(),
                                      c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
@@ -646,14 +678,12 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
         // lists without the cap and blends again.  The work is enqueued now
         // and gated on the blend's flag, so the host never waits for it.
         stage_begin(c, "list_refill", st);
-        UPS_CUDA(c, bucket_sort_u32(ik, iv, iv_alt, n_inst, vt.total_tiles, kNoListCap, c->ranges.as<uint2>(),
-                                    c->trunc.as<uint32_t>(), c->sort.hist.ptr, c->sort.hist.bytes, c->num_sms, st,
-                                    c->d_trunc_flag));
+        UPS_CUDA(c, lists(kNoListCap, c->d_trunc_flag));
         UPS_CUDA(c, launch_composite_fwd(vt, c->bp, c->cfg.n_feat, c->N, c->per_view, c->ranges.as<uint2>(),
                                          c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
                                          reinterpret_cast<const float4 *>(g->color), g->feat, *out, st, nullptr,
                                          nullptr, c->d_trunc_flag, c->d_err));
-        stage_end(c, st, 7);
+        stage_end(c, st, 3);
     }
     c->g_in = *g;
     c->img = *out;
@@ -1025,6 +1055,7 @@ ups_status ups_copy_buffer(ups_ctx *c, int which, void *dst, size_t bytes, size_
             sz = listed * 4;
             if (!c->ikey_sorted && sz) {
                 UPS_CUDA(c, cudaSetDevice(c->device));
+                UPS_CUDA(c, c->ikey1.reserve(sz));
                 UPS_CUDA(c, keys_from_ranges(c->ranges.as<uint2>(), c->vt.total_tiles, c->ikey1.as<uint32_t>(),
                                              c->last_stream));
                 c->ikey_sorted = c->ikey1.as<uint32_t>();

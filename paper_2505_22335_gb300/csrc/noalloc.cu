@@ -33,10 +33,9 @@
 
 namespace ups {
 
-cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                           int total, const ups_gaussians &g, float4 *xyzo, float4 *conic,
-                           uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
-                           cudaStream_t st);
+cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
+                           float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
+                           uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
 cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *count, uint32_t *out,
                                  int total, cudaStream_t st);
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
@@ -210,7 +209,7 @@ extern "C" ups_status ups_render_forward_static(const ups_config *cfg, const ups
     void *sort_scr = base + oSort;
     void *scan_scr = base + oScan;
 
-    NA_CUDA(launch_project(vt, bp, N, per_view, (int)total, *g, xyzo, conic, rect, count, dk, dv, st));
+    NA_CUDA(launch_project(vt, bp, N, (int)total, *g, xyzo, conic, rect, count, dk, dv, nullptr, nullptr, nullptr, st));
     NA_CUDA(radix_sort_u64_fixed(&dk, &dk_alt, &dv, &dv_alt, total, 32 + bits_for((size_t)n_views),
                                  sort_scr, kSortScratch, st));
     NA_CUDA(launch_gather_counts(dv, count, cnt, (int)total, st));

@@ -1,9 +1,10 @@
-// EWA projection of 3D Gaussians (Eq. 1-2), depth keys, tile-instance
-// emission and tile ranges, and the projection backward into mean, scale,
+// EWA projection of 3D Gaussians (Eq. 1-2), depth keys, packed tile spans, tile-
+// instance emission and tile ranges (for views too large for the row-wise lists), and the projection backward into mean, scale,
 // rotation and SE(3) pose gradients.
 //
 // One thread per Gaussian-view; attributes are read as float4 records.
 #include "common.cuh"
+#include "tiles.cuh"
 
 namespace ups {
 
@@ -92,120 +93,170 @@ __device__ __forceinline__ void covariance(const DevView &cam, const BlendParams
     G.C = t1[0] * G.T[3] + t1[1] * G.T[4] + t1[2] * G.T[5] + bp.dilation;
 }
 
-// The alpha >= alpha_min ellipse q(d) = a dx^2 + 2 b dx dy + c dy^2 <= k2,
-// k2 = 2 ln(o / alpha_min), of a projected Gaussian at (u, v), conic (a, b, c).
-// Tile decisions use a margin so that FP32 rounding never drops a tile the
-// blend uses: k2 grown by kMarginQ (relative) and every tile's box of pixel
-// centres grown by kMarginPx on each side; the rectangle is the box of that
-// grown ellipse, grown by kMarginPx.  A list may thus hold, besides the exact
-// tiles, tiles whose box the exact ellipse misses by less than the margin.
-constexpr float kMarginQ = 1e-4f;
-constexpr float kMarginPx = 1e-3f;
+// One Gaussian-view per thread: projection, depth key and tile rectangle; then
+// the tiles it meets, row by row.  A Gaussian meets 1 to over 20 tile rows, and
+// a row costs two square roots and a division, so the rows are spread over the
+// warp: lane i of a step takes the i-th (Gaussian, row) of the warp and reads
+// that Gaussian's ellipse by shuffle (issue-bound: 78 % issue active; the
+// per-thread loop ran with 17 of 32 lanes on and took 0.33 ms for 8M Gaussian-
+// views at 640x480 and 0.44 at 1280x720 with the packed spans, this form 0.29
+// and 0.34; without spans the loop took 0.24 and 0.30).  Row codes are collected in shared memory and
+// packed by the owning thread (span and more may be null: counts only).
+constexpr int kProjThreads = 256;
 
-struct Ellipse {
-    float u, v, a, b, k2, detc, ry, dyr;
-};
-
-__device__ __forceinline__ Ellipse ellipse_of(float4 xo, float4 cn, float alpha_min) {
-    Ellipse e;
-    e.u = xo.x;
-    e.v = xo.y;
-    e.a = cn.x;
-    e.b = cn.y;
-    // a relative margin so FP32 rounding never drops a tile the blend uses
-    e.k2 = 2.f * logf(xo.w / alpha_min) * (1.f + kMarginQ);
-    e.detc = cn.x * cn.z - cn.y * cn.y;
-    e.ry = sqrtf(e.k2 * cn.x / e.detc);               // half-extent in y
-    e.dyr = -cn.y * sqrtf(e.k2 / (cn.z * e.detc));    // dy of the point of largest x
-    return e;
-}
-
-// Tile columns [c0, c1] of tile row ty (clipped to the rect's columns
-// [x0, x1]; c0 > c1: none) whose box of pixel centres the ellipse meets.  The
-// ellipse's slice through the row's band of pixel centres is an x interval;
-// its ends are the right-most and left-most boundary points, whose dy is the
-// unconstrained extreme clamped to the band (the boundary's x is concave /
-// convex in dy).
-__device__ __forceinline__ int2 row_cols(const Ellipse &e, int ty, int W, int H, int x0, int x1) {
-    const float yb0 = (float)(ty * kTile) - kMarginPx,
-                yb1 = fminf((float)(ty * kTile + kTile - 1), (float)(H - 1)) + kMarginPx;
-    const float lo = fmaxf(yb0 - e.v, -e.ry), hi = fminf(yb1 - e.v, e.ry);
-    if (!(lo <= hi)) return make_int2(1, 0);
-    const float dr = fminf(fmaxf(e.dyr, lo), hi), dl = fminf(fmaxf(-e.dyr, lo), hi);
-    const float ia = 1.f / e.a;
-    const float xr = (-e.b * dr + sqrtf(fmaxf(e.a * e.k2 - e.detc * dr * dr, 0.f))) * ia;
-    const float xl = (-e.b * dl - sqrtf(fmaxf(e.a * e.k2 - e.detc * dl * dl, 0.f))) * ia;
-    const float xlo = fmaxf(e.u + xl - kMarginPx, 0.f), xhi = fminf(e.u + xr + kMarginPx, (float)(W - 1));
-    if (!(xlo <= xhi)) return make_int2(1, 0);
-    // tile tx holds pixel centres [16 tx, 16 tx + 15]: the first whose box
-    // reaches xlo, the last whose box starts at or before xhi
-    return make_int2(max((int)ceilf((xlo - (float)(kTile - 1)) * (1.f / kTile)), x0),
-                     min((int)floorf(xhi * (1.f / kTile)), x1));
-}
-
-__global__ void __launch_bounds__(256) k_project(
-    ViewTable vt, BlendParams bp, int N, int per_view, int total,
-    const float4 *__restrict__ mean_op, const float4 *__restrict__ scale,
-    const float4 *__restrict__ quat, float4 *__restrict__ xyzo, float4 *__restrict__ conic,
-    uint2 *__restrict__ rect, uint32_t *__restrict__ count, uint64_t *__restrict__ dkey,
-    uint32_t *__restrict__ dval, uint32_t *__restrict__ dkey32, int vbits32) {
-    int gv = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gv >= total) return;
-    int v = gv / N;
+__global__ void __launch_bounds__(kProjThreads) k_project(
+    ViewTable vt, BlendParams bp, int N, const float4 *__restrict__ mean_op,
+    const float4 *__restrict__ scale, const float4 *__restrict__ quat, float4 *__restrict__ xyzo,
+    float4 *__restrict__ conic, uint2 *__restrict__ rect, uint32_t *__restrict__ count,
+    uint64_t *__restrict__ dkey, uint32_t *__restrict__ dval, uint32_t *__restrict__ dkey32, int vbits32,
+    uint4 *__restrict__ span, uint4 *__restrict__ more, unsigned long long *__restrict__ n_inst) {
+    __shared__ uint16_t s_code[kSpanRows][kProjThreads];  // columns after x0 | count << 8
+    __shared__ uint32_t s_cnt[kProjThreads];              // tiles met in rows that have no code
+    __shared__ uint8_t s_own[kProjThreads];               // a warp's lanes that have rows, in order
+    __shared__ uint32_t s_wide[kProjThreads / 32];        // lanes with a row that does not fit a code
+    __shared__ uint32_t wsum[kProjThreads / 32];
+    const unsigned full = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int v = blockIdx.y, gi = blockIdx.x * kProjThreads + tid, gv = v * N + gi;
+    const bool in = gi < N;
     const DevView &cam = vt.v[v];
-    int gs = cam.set * N + (gv - v * N);
-    float4 m = mean_op[gs];
-    Geo G;
-    bool ok = camera_point(cam, bp, m, G.p);
-    uint32_t cnt = 0;
     uint2 rc = make_uint2(0u, 0u);
-    float4 xo = make_float4(0.f, 0.f, G.p[2], m.w);
-    float4 cn = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (ok) {
-        covariance(cam, bp, scale[gs], quat[gs], G);
-        float det = G.A * G.C - G.B * G.B;
-        float idet = 1.f / det;
-        cn = make_float4(G.C * idet, -G.B * idet, G.A * idet, 0.f);
-        float iz = 1.f / G.p[2];
-        float u = fmaf(cam.fx * G.p[0], iz, cam.cx);
-        float vv = fmaf(cam.fy * G.p[1], iz, cam.cy);
-        xo.x = u;
-        xo.y = vv;
-        // bounding box of the ellipse o exp(-q/2) >= alpha_min, with the
-        // margin of the tile decisions
-        float k2 = 2.f * logf(m.w / bp.alpha_min) * (1.f + kMarginQ);
-        float rx = sqrtf(k2 * G.A) + kMarginPx, ry = sqrtf(k2 * G.C) + kMarginPx;
-        float xlo = fmaxf(u - rx, 0.f), xhi = fminf(u + rx, (float)(cam.W - 1));
-        float ylo = fmaxf(vv - ry, 0.f), yhi = fminf(vv + ry, (float)(cam.H - 1));
-        if (xlo <= xhi && ylo <= yhi) {
-            int x0 = (int)floorf(xlo * (1.f / kTile)), x1 = (int)floorf(xhi * (1.f / kTile));
-            int y0 = (int)floorf(ylo * (1.f / kTile)), y1 = (int)floorf(yhi * (1.f / kTile));
-            // tiles of the rect that the ellipse meets (same arithmetic as k_emit)
-            const Ellipse e = ellipse_of(xo, cn, bp.alpha_min);
-            for (int ty = y0; ty <= y1; ++ty) {
-                const int2 cc = row_cols(e, ty, cam.W, cam.H, x0, x1);
-                if (cc.x <= cc.y) cnt += (uint32_t)(cc.y - cc.x + 1);
+    float4 xo = make_float4(0.f, 0.f, 0.f, 0.f), cn = xo;
+    Ellipse e{};
+    int nrow = 0;
+    float z = 0.f;
+    if (in) {
+        int gs = cam.set * N + gi;
+        float4 m = mean_op[gs];
+        Geo G;
+        bool ok = camera_point(cam, bp, m, G.p);
+        z = G.p[2];
+        xo = make_float4(0.f, 0.f, G.p[2], m.w);
+        if (ok) {
+            covariance(cam, bp, scale[gs], quat[gs], G);
+            float det = G.A * G.C - G.B * G.B;
+            float idet = 1.f / det;
+            cn = make_float4(G.C * idet, -G.B * idet, G.A * idet, 0.f);
+            float iz = 1.f / G.p[2];
+            float u = fmaf(cam.fx * G.p[0], iz, cam.cx);
+            float vv = fmaf(cam.fy * G.p[1], iz, cam.cy);
+            xo.x = u;
+            xo.y = vv;
+            // bounding box of the ellipse o exp(-q/2) >= alpha_min, with the
+            // margin of the tile decisions
+            float k2 = 2.f * logf(m.w / bp.alpha_min) * (1.f + kMarginQ);
+            float rx = sqrtf(k2 * G.A) + kMarginPx, ry = sqrtf(k2 * G.C) + kMarginPx;
+            float xlo = fmaxf(u - rx, 0.f), xhi = fminf(u + rx, (float)(cam.W - 1));
+            float ylo = fmaxf(vv - ry, 0.f), yhi = fminf(vv + ry, (float)(cam.H - 1));
+            if (xlo <= xhi && ylo <= yhi) {
+                int x0 = (int)floorf(xlo * (1.f / kTile)), x1 = (int)floorf(xhi * (1.f / kTile));
+                int y0 = (int)floorf(ylo * (1.f / kTile)), y1 = (int)floorf(yhi * (1.f / kTile));
+                e = ellipse_of(xo, cn, bp.alpha_min);
+                rc = make_uint2((uint32_t)x0 | ((uint32_t)y0 << 16), (uint32_t)x1 | ((uint32_t)y1 << 16));
+                nrow = y1 - y0 + 1;
             }
-            rc = make_uint2((uint32_t)x0 | ((uint32_t)y0 << 16), (uint32_t)x1 | ((uint32_t)y1 << 16));
+        }
+        xyzo[gv] = xo;
+        conic[gv] = cn;
+        rect[gv] = rc;
+    }
+    s_cnt[tid] = 0u;
+    if (lane == 0) s_wide[wid] = 0u;
+    int incl = nrow;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(full, incl, o);
+        if (lane >= o) incl += y;
+    }
+    const int rows = __shfl_sync(full, incl, 31), first = incl - nrow;
+    const uint32_t some = __ballot_sync(full, nrow > 0);
+    if (nrow > 0) s_own[(wid << 5) + __popc(some & ((1u << lane) - 1u))] = (uint8_t)lane;
+    __syncwarp();
+    int before = 0;  // owners whose rows start before the step
+    for (int b = 0; b < rows; b += 32) {
+        const int i = b + lane;
+        // the owner of row i: the last whose rows start at or before it
+        const uint32_t starts =
+            __reduce_or_sync(full, nrow > 0 && first >= b && first < b + 32 ? 1u << (first - b) : 0u);
+        const int L = s_own[(wid << 5) + before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1];
+        before += __popc(starts);
+        Ellipse t;
+        t.u = __shfl_sync(full, e.u, L);
+        t.v = __shfl_sync(full, e.v, L);
+        t.a = __shfl_sync(full, e.a, L);
+        t.b = __shfl_sync(full, e.b, L);
+        t.k2 = __shfl_sync(full, e.k2, L);
+        t.detc = __shfl_sync(full, e.detc, L);
+        t.ry = __shfl_sync(full, e.ry, L);
+        t.dyr = __shfl_sync(full, e.dyr, L);
+        t.ia = __shfl_sync(full, e.ia, L);
+        const uint32_t r0 = __shfl_sync(full, rc.x, L), r1 = __shfl_sync(full, rc.y, L);
+        const int k = i - __shfl_sync(full, first, L);
+        if (i < rows) {
+            const int x0 = r0 & 0xffff, x1 = r1 & 0xffff;
+            const int2 cc = row_cols(t, (int)(r0 >> 16) + k, cam.W, cam.H, x0, x1);
+            const int off = cc.x - x0, len = cc.x <= cc.y ? cc.y - cc.x + 1 : 0;
+            const bool coded = k < kSpanRows && off <= 255 && len <= 255;
+            if (k < kSpanRows) s_code[k][(wid << 5) + L] = coded && len ? (uint16_t)(off | (len << 8)) : (uint16_t)0;
+            if (len && !coded) {
+                atomicAdd(&s_cnt[(wid << 5) + L], (uint32_t)len);
+                if (k < kSpanRows) atomicOr(&s_wide[wid], 1u << L);
+            }
         }
     }
-    xyzo[gv] = xo;
-    conic[gv] = cn;
-    rect[gv] = rc;
-    count[gv] = cnt;
-    if (vbits32 < 0) {
-        uint32_t zb = cnt ? __float_as_uint(G.p[2]) : 0xffffffffu;
-        dkey[gv] = ((uint64_t)v << 32) | zb;
-    } else {
-        // 32-bit key: view in the top vbits32 bits, float bits of z above
-        // 0.125 m below (exact while z < 2^(32 - vbits32) ulps above 0.125 m;
-        // larger depths saturate and fall back to id order)
-        const uint32_t zmask = vbits32 == 0 ? 0xffffffffu : (0xffffffffu >> vbits32);
-        uint32_t zf = zmask;
-        if (cnt) zf = min(__float_as_uint(G.p[2]) - 0x3e000000u, zmask);
-        dkey32[gv] = (vbits32 == 0 ? 0u : ((uint32_t)v << (32 - vbits32))) | zf;
+    __syncwarp();
+    uint32_t cnt = s_cnt[tid];
+    uint32_t pair[kSpanRows / 2];  // two rows a word
+#pragma unroll
+    for (int k = 0; k < kSpanRows; k += 2) {
+        pair[k / 2] = 0u;
+        if (k >= nrow) continue;
+        const uint32_t lo = s_code[k][tid], hi = k + 1 < nrow ? s_code[k + 1][tid] : 0u;
+        pair[k / 2] = lo | (hi << 16);
+        cnt += (lo >> 8) + (hi >> 8);
     }
-    dval[gv] = (uint32_t)gv;
+    if (in) {
+        count[gv] = cnt;
+        if (span) {
+            const uint32_t head = (rc.x & 1023u) | ((rc.x >> 16 & 1023u) << 10) |
+                                  (min((rc.y & 0xffffu) - (rc.x & 0xffffu), kSpanWide) << 25);
+            uint4 s = make_uint4(0u, 0u, 0u, 0u);
+            if (cnt && (nrow > kSpanRows || (s_wide[wid] >> lane & 1u))) {
+                s = make_uint4(head | (kSpanTall << 20), rc.x, rc.y, 0u);
+            } else if (cnt) {
+                s = make_uint4(head | ((uint32_t)nrow << 20), pair[0], pair[1], pair[2]);
+                uint4 *m = more + (size_t)kSpanMore * gv;
+                if (nrow > kSpanRows1) m[0] = make_uint4(pair[3], pair[4], pair[5], pair[6]);
+                if (nrow > kSpanRows1 + 8) m[1] = make_uint4(pair[7], pair[8], pair[9], pair[10]);
+            }
+            span[gv] = s;
+        }
+        if (vbits32 < 0) {
+            uint32_t zb = cnt ? __float_as_uint(z) : 0xffffffffu;
+            dkey[gv] = ((uint64_t)v << 32) | zb;
+        } else {
+            // 32-bit key: view in the top vbits32 bits, float bits of z above
+            // 0.125 m below (exact while z < 2^(32 - vbits32) ulps above 0.125 m;
+            // larger depths saturate and fall back to id order)
+            const uint32_t zmask = vbits32 == 0 ? 0xffffffffu : (0xffffffffu >> vbits32);
+            uint32_t zf = zmask;
+            if (cnt) zf = min(__float_as_uint(z) - 0x3e000000u, zmask);
+            dkey32[gv] = (vbits32 == 0 ? 0u : ((uint32_t)v << (32 - vbits32))) | zf;
+        }
+        dval[gv] = (uint32_t)gv;
+    }
+    if (!n_inst) return;
+    // tile instances for the host's total: one atomic a block, spread over
+    // kInstCounters addresses so that 31,250 blocks (8M Gaussian-views) do not
+    // queue up at one
+    const uint32_t ws = __reduce_add_sync(full, cnt);
+    if (lane == 0) wsum[wid] = ws;
+    __syncthreads();
+    if (tid == 0) {
+        unsigned long long s = 0;
+        for (int w = 0; w < kProjThreads / 32; ++w) s += wsum[w];
+        if (s) atomicAdd(n_inst + (blockIdx.x + blockIdx.y) % kInstCounters, s);
+    }
 }
 
 __global__ void k_gather_counts(const uint32_t *__restrict__ sorted_gv,
@@ -538,28 +589,26 @@ __global__ void __launch_bounds__(256) k_project_bwd(
 
 }  // namespace
 
-cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                           int total, const ups_gaussians &g, float4 *xyzo, float4 *conic,
-                           uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
-                           cudaStream_t st) {
+cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
+                           float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint64_t *dkey, uint32_t *dval,
+                           uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st) {
     if (total == 0) return cudaSuccess;
-    k_project<<<(total + 255) / 256, 256, 0, st>>>(
-        vt, bp, N, per_view, total, reinterpret_cast<const float4 *>(g.mean_opacity),
+    k_project<<<dim3((N + kProjThreads - 1) / kProjThreads, vt.n), kProjThreads, 0, st>>>(
+        vt, bp, N, reinterpret_cast<const float4 *>(g.mean_opacity),
         reinterpret_cast<const float4 *>(g.scale), reinterpret_cast<const float4 *>(g.quat), xyzo,
-        conic, rect, count, dkey, dval, nullptr, -1);
+        conic, rect, count, dkey, dval, nullptr, -1, span, more, n_inst);
     return cudaGetLastError();
 }
 
 // Projection writing 32-bit (view, depth) keys (vbits = bits of the view index).
-cudaError_t launch_project_k32(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                               int total, const ups_gaussians &g, float4 *xyzo, float4 *conic,
-                               uint2 *rect, uint32_t *count, uint32_t *dkey32, uint32_t *dval,
-                               int vbits, cudaStream_t st) {
+cudaError_t launch_project_k32(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
+                               float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint32_t *dkey32,
+                               uint32_t *dval, int vbits, uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st) {
     if (total == 0) return cudaSuccess;
-    k_project<<<(total + 255) / 256, 256, 0, st>>>(
-        vt, bp, N, per_view, total, reinterpret_cast<const float4 *>(g.mean_opacity),
+    k_project<<<dim3((N + kProjThreads - 1) / kProjThreads, vt.n), kProjThreads, 0, st>>>(
+        vt, bp, N, reinterpret_cast<const float4 *>(g.mean_opacity),
         reinterpret_cast<const float4 *>(g.scale), reinterpret_cast<const float4 *>(g.quat), xyzo,
-        conic, rect, count, nullptr, dval, dkey32, vbits);
+        conic, rect, count, nullptr, dval, dkey32, vbits, span, more, n_inst);
     return cudaGetLastError();
 }
 
