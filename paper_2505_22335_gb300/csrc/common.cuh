@@ -45,6 +45,12 @@ struct BlendParams {
 constexpr int kG2Base = 12;
 __host__ __device__ inline int g2_stride(int n_feat) { return kG2Base + n_feat; }
 
+// The Gaussian-views that a blend backward staged: a bit each, then each id once
+// and their number.
+struct HitList {
+    uint32_t *bits, *list, *count;
+};
+
 // View index of global tile `t` (views are few; linear scan).
 __device__ __forceinline__ int view_of_tile(const ViewTable &vt, int t) {
     int v = 0;

@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
     const float *__restrict__ feat, const float *__restrict__ in_T,
     const uint32_t *__restrict__ in_nc, const float *__restrict__ dC,
     const float *__restrict__ dD, const float *__restrict__ dF, const float *__restrict__ dT,
-    float *__restrict__ g2, int *__restrict__ err) {
+    float *__restrict__ g2, uint32_t *__restrict__ hits, int *__restrict__ err) {
     constexpr int NT = Px<PX>::NT, RS = Px<PX>::RS, NW = NT / 32, NS = kBwdStages;
     constexpr int KB = NF > 16 ? 32 : UPS_BWD_BATCH;
     constexpr int STRIDE = kG2Base + NF;  // record floats, a multiple of 4
@@ -517,7 +517,10 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
         const int lo = lo_of(b), cnt = max_nc - b * KB - lo;
         Stage<NF, KB> &S = ring[b % NS];
         if (tid == 0) mbar_expect(&mbar[b % NS], (uint32_t)cnt * StageBytes<NF>::value);
-        if (tid < cnt) stage_entry<NF, KB>(S, tid, gv, (int)gv - set_base, xyzo, conic, color, feat, &mbar[b % NS]);
+        if (tid < cnt) {
+            stage_entry<NF, KB>(S, tid, gv, (int)gv - set_base, xyzo, conic, color, feat, &mbar[b % NS]);
+            atomicOr(hits + (gv >> 5), 1u << (gv & 31u));  // its gradient record may be written
+        }
     };
     int issued = min(NS, nb);
     {
@@ -698,12 +701,13 @@ cudaError_t launch_composite_bwd(const ViewTable &vt, const BlendParams &bp, int
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
                                  const float *feat, const float *T, const uint32_t *nc,
-                                 const ups_image_grads &dL, float *g2, cudaStream_t st, int *err) {
+                                 const ups_image_grads &dL, float *g2, uint32_t *hits, cudaStream_t st,
+                                 int *err) {
     if (vt.total_tiles == 0) return cudaSuccess;
 #define UPS_BWD(NFV)                                                                                \
     k_composite_bwd<NFV, blend_px_bwd(NFV)><<<vt.total_tiles, Px<blend_px_bwd(NFV)>::NT, 0, st>>>(            \
         vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, T, nc, dL.color, dL.depth, dL.feat, \
-        dL.T, g2, err)
+        dL.T, g2, hits, err)
     switch (n_feat) {
         case 0: UPS_BWD(0); break;
         case 16: UPS_BWD(16); break;

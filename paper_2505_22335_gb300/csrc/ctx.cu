@@ -28,10 +28,12 @@ cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int t
                         const uint64_t *off, const uint2 *rect, const float4 *xyzo, const float4 *conic,
                         uint32_t *ikey, uint32_t *ival, cudaStream_t st);
 cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaStream_t st);
-cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                               int total, int n_feat, unsigned mask, float scale_grad,
-                               const ups_gaussians &g, const float *g2, const ups_gaussians *grad,
-                               float *d_pose, cudaStream_t st);
+cudaError_t launch_clear_hits(const HitList &hits, size_t n_gv, float *g2, int n_feat, int num_sms, cudaStream_t st);
+cudaError_t launch_list_hits(const HitList &hits, size_t n_gv, cudaStream_t st);
+cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N, int n_sets, int direct, int n_feat,
+                               unsigned mask, float scale_grad, const ups_gaussians &g, const float *g2,
+                               const HitList &hits, const ups_gaussians *grad, float *d_pose, int num_sms,
+                               cudaStream_t st);
 cudaError_t launch_composite_fwd(const ViewTable &vt, const BlendParams &bp, int n_feat, int N,
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
@@ -70,7 +72,8 @@ cudaError_t launch_composite_bwd(const ViewTable &vt, const BlendParams &bp, int
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
                                  const float *feat, const float *T, const uint32_t *nc,
-                                 const ups_image_grads &dL, float *g2, cudaStream_t st, int *err);
+                                 const ups_image_grads &dL, float *g2, uint32_t *hits, cudaStream_t st,
+                                 int *err);
 cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const ups_anchors &anc,
                               const ups_mlp &mlp, const ups_gaussians &out, int op_tanh, int num_sms,
                               cudaStream_t st);
@@ -128,8 +131,12 @@ struct ups_ctx {
     ups_gaussians g_in{};
     ups_images img{};
     bool have_bwd = false;
+    // gradient records g2 and the list of those the last backward staged (below
+    // g2_used): once g2_known every record that is not listed is zero
+    bool g2_known = false;
+    size_t g2_used = 0;
     // scratch
-    DevBuf xyzo, conic, rect, count, span, more, dkey0, dkey1, dval0, dval1, bin_scr, lists, ranges, g2;
+    DevBuf xyzo, conic, rect, count, span, more, dkey0, dkey1, dval0, dval1, bin_scr, lists, ranges, g2, hit_bits, hit_list;
     // views too large for the row-wise tile lists: instances, their offsets and sort buffers
     DevBuf cnt_sorted, off, scan_scr, ikey0, ikey1, ival0, ival1;
     DevBuf dec_scratch;  // decode backward: X, H, dL/dY, dL/dZ rows for the weight gradients
@@ -141,6 +148,7 @@ struct ups_ctx {
         unsigned long long n_inst[kInstCounters];
         int trunc_flag;  // set by the forward blend: a capped list was too short
         int err;         // set by kernels whose bounded waits ran out
+        uint32_t n_hits; // length of the last backward's hit list
     };
     Words *d_words = nullptr, *h_words = nullptr;
     cudaEvent_t words_ready = nullptr;  // the pinned copy has arrived
@@ -467,7 +475,7 @@ ups_status ups_destroy(ups_ctx *c) {
     cudaSetDevice(c->device);
     DevBuf *bufs[] = {&c->xyzo, &c->conic, &c->rect, &c->count, &c->span, &c->more, &c->bin_scr, &c->lists, &c->dkey0,
                       &c->dkey1, &c->dval0, &c->dval1, &c->cnt_sorted, &c->off, &c->scan_scr, &c->ikey0, &c->ikey1,
-                      &c->ival0, &c->ival1, &c->ranges, &c->g2, &c->dec_scratch, &c->sort.hist, &c->trunc, &c->lift_scr, &c->ssim_g, &c->unc_scr, &c->anchor_scr};
+                      &c->ival0, &c->ival1, &c->ranges, &c->g2, &c->hit_bits, &c->hit_list, &c->dec_scratch, &c->sort.hist, &c->trunc, &c->lift_scr, &c->ssim_g, &c->unc_scr, &c->anchor_scr};
     for (DevBuf *b : bufs) b->release();
     if (c->h_words) cudaFreeHost(c->h_words);
     if (c->h_anchor) cudaFreeHost(c->h_anchor);
@@ -936,14 +944,38 @@ ups_status ups_render_backward(ups_ctx *c, const ups_image_grads *dL, unsigned m
     c->last_stream = st;
     const int nf = c->cfg.n_feat;
     const size_t rec = (size_t)g2_stride(nf);
-    UPS_CUDA(c, c->g2.reserve(c->total_gv * rec * sizeof(float)));
-    UPS_CUDA(c, cudaMemsetAsync(c->g2.ptr, 0, c->total_gv * rec * sizeof(float), st));
+    // zero records: those that the last backward staged are cleared, new buffers
+    // (or ones left by a failed call) whole
+    const size_t g2_bytes = c->total_gv * rec * sizeof(float), bit_bytes = (c->total_gv + 31) / 32 * 4;
+    if (g2_bytes > c->g2.bytes || bit_bytes > c->hit_bits.bytes || c->total_gv * 4 > c->hit_list.bytes) {
+        c->g2_known = false;
+        UPS_CUDA(c, c->g2.reserve(g2_bytes));
+        UPS_CUDA(c, c->hit_bits.reserve(bit_bytes));
+        UPS_CUDA(c, c->hit_list.reserve(c->total_gv * 4));
+    }
+    const HitList hits{c->hit_bits.as<uint32_t>(), c->hit_list.as<uint32_t>(), &c->d_words->n_hits};
+    const bool known = c->g2_known;
+    c->g2_known = false;
+    stage_begin(c, "clear_records", st);
+    if (known) {
+        UPS_CUDA(c, launch_clear_hits(hits, c->g2_used, c->g2.as<float>(), nf, c->num_sms, st));
+    } else {
+        UPS_CUDA(c, cudaMemsetAsync(c->g2.ptr, 0, c->g2.bytes, st));
+        UPS_CUDA(c, cudaMemsetAsync(c->hit_bits.ptr, 0, c->hit_bits.bytes, st));
+    }
+    UPS_CUDA(c, cudaMemsetAsync(hits.count, 0, sizeof(uint32_t), st));
+    stage_end(c, st, known ? 1 : 0);
     stage_begin(c, "composite_bwd", st);
     UPS_CUDA(c, launch_composite_bwd(c->vt, c->bp, nf, c->N, c->per_view, c->ranges.as<uint2>(),
                                      c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
                                      reinterpret_cast<const float4 *>(c->g_in.color), c->g_in.feat,
-                                     c->img.T, c->img.n_contrib, *dL, c->g2.as<float>(), st, c->d_err));
+                                     c->img.T, c->img.n_contrib, *dL, c->g2.as<float>(),
+                                     hits.bits, st, c->d_err));
     stage_end(c, st, 1);
+    UPS_CUDA(c, launch_list_hits(hits, c->total_gv, st));
+    c->launches += 1;
+    c->g2_known = true;
+    c->g2_used = c->total_gv;
     if (mask & UPS_GRAD_POSE)
         UPS_CUDA(c, cudaMemsetAsync(d_pose, 0, sizeof(float) * 6 * c->vt.n, st));
     if ((mask & UPS_GRAD_GAUSS) && c->shared_sets) {
@@ -956,9 +988,9 @@ ups_status ups_render_backward(ups_ctx *c, const ups_image_grads *dL, unsigned m
     }
     if (mask & (UPS_GRAD_POSE | UPS_GRAD_GAUSS)) {
         stage_begin(c, "project_bwd", st);
-        UPS_CUDA(c, launch_project_bwd(c->vt, c->bp, c->N, c->shared_sets ? 0 : 1, (int)c->total_gv, nf, mask,
-                                       scale_grad, c->g_in, c->g2.as<float>(), grad, d_pose, st));
-        stage_end(c, st, 1);
+        UPS_CUDA(c, launch_project_bwd(c->vt, c->bp, c->N, c->n_sets, c->shared_sets ? 0 : 1, nf, mask, scale_grad,
+                                       c->g_in, c->g2.as<float>(), hits, grad, d_pose, c->num_sms, st));
+        stage_end(c, st, (mask & UPS_GRAD_GAUSS) && (!c->shared_sets || scale_grad != 0.f) ? 2 : 1);
     }
     c->have_bwd = true;
     return UPS_OK;

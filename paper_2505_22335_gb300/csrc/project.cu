@@ -3,6 +3,8 @@
 // rotation and SE(3) pose gradients.
 //
 // One thread per Gaussian-view; attributes are read as float4 records.
+#include <algorithm>
+
 #include "common.cuh"
 #include "tiles.cuh"
 
@@ -373,28 +375,76 @@ __global__ void k_ranges(const uint32_t *__restrict__ ikey, uint32_t n, uint2 *_
 // backward
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(256) k_project_bwd(
-    ViewTable vt, BlendParams bp, int N, int direct, int total, int n_feat, unsigned mask,
+// The blend backward sets a bit for every Gaussian-view it stages; only those
+// have a gradient record that can differ from zero.  At 1M Gaussians and 8 x
+// 640x480 it stages 1.6M list entries, a few percent of the 8M Gaussian-views,
+// so the projection backward is a zero fill of the gradients, bound by its
+// writes (128 B a Gaussian-view at 16 channels), and this kernel over the list
+// of set bits (k_list_hits), one Gaussian-view a thread of a grid-stride loop:
+// 0.19 ms and 0.01 to clear the records.  A thread per Gaussian-view reading
+// every record took 0.47 ms after a 0.14 ms memset of the records; skipping
+// those without a flag 0.31 ms (nearly every warp had a lane to evaluate), as
+// did CTAs that list the bits of their own words (too few lanes busy); a list
+// appended by the blend kernel cost that kernel 0.03 ms of atomic latency.
+constexpr int kBwdThreads = 256;
+
+// hits.list = the set bits' Gaussian-views (in order inside a CTA's words);
+// *hits.count was zero
+__global__ void __launch_bounds__(256) k_list_hits(HitList hits, size_t n_words) {
+    __shared__ uint32_t wsum[8];
+    __shared__ uint32_t s_at;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;
+    uint32_t b = w < n_words ? hits.bits[w] : 0u;
+    uint32_t incl = __popc(b);
+    const uint32_t c = incl;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) wsum[wid] = incl;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        before += i < wid ? wsum[i] : 0u;
+        all += wsum[i];
+    }
+    if (all == 0) return;
+    if (threadIdx.x == 0) s_at = atomicAdd(hits.count, all);
+    __syncthreads();
+    for (uint32_t at = s_at + before + incl - c; b; b &= b - 1) hits.list[at++] = (uint32_t)(32 * w) + __ffs(b) - 1;
+}
+
+__global__ void __launch_bounds__(kBwdThreads) k_project_bwd(
+    ViewTable vt, BlendParams bp, int N, int direct, int n_feat, unsigned mask,
     float scale_grad, const float4 *__restrict__ mean_op, const float4 *__restrict__ scale,
-    const float4 *__restrict__ quat, const float *__restrict__ g2, float4 *__restrict__ d_mean_op,
-    float4 *__restrict__ d_scale, float4 *__restrict__ d_quat, float4 *__restrict__ d_color,
-    float *__restrict__ d_feat, float *__restrict__ d_pose) {
-    int gv = blockIdx.x * blockDim.x + threadIdx.x;
-    bool in = gv < total;
-    int v = in ? gv / N : vt.n - 1;
-    // direct: every set is read by one view, so its gradient is written, not
-    // accumulated (else the caller zeroed the gradient and views add into it)
-    int gs = vt.v[v].set * N + (gv - v * N);
-    float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (in) {
+    const float4 *__restrict__ quat, const float *__restrict__ g2, HitList hits,
+    float4 *__restrict__ d_mean_op, float4 *__restrict__ d_scale, float4 *__restrict__ d_quat,
+    float4 *__restrict__ d_color, float *__restrict__ d_feat, float *__restrict__ d_pose) {
+    const unsigned full = 0xffffffffu;
+    __shared__ float s_pose[UPS_MAX_VIEWS][6];
+    for (int i = threadIdx.x; i < 6 * vt.n; i += kBwdThreads) (&s_pose[0][0])[i] = 0.f;
+    __syncthreads();
+    const int stride = g2_stride(n_feat), lane = threadIdx.x & 31;
+    const size_t n_hits = *hits.count;
+    for (size_t i0 = (size_t)blockIdx.x * kBwdThreads + threadIdx.x - lane; i0 < n_hits;
+         i0 += (size_t)gridDim.x * kBwdThreads) {
+        const bool in = i0 + lane < n_hits;
+        const size_t gv = in ? hits.list[i0 + lane] : 0u;
+        const int v = (int)(gv / (unsigned)N);
         const DevView &cam = vt.v[v];
-        float4 m = mean_op[gs];
-        Geo G;
-        bool ok = camera_point(cam, bp, m, G.p);
-        const int stride = g2_stride(n_feat);
-        const float *r = g2 + (size_t)gv * stride;
+        // direct: every set is read by one view, so its gradient is written, not
+        // accumulated (else the caller zeroed the gradient and views add into it)
+        const size_t gs = (size_t)cam.set * N + (gv - (size_t)v * N);
+        const float *r = g2 + gv * stride;
+        float pose[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         float dmu[3] = {0.f, 0.f, 0.f}, ds[3] = {0.f, 0.f, 0.f}, dq[4] = {0.f, 0.f, 0.f, 0.f};
         float dop = 0.f;
+        bool ok = false;
+        Geo G;
+        if (in) ok = camera_point(cam, bp, mean_op[gs], G.p);
         if (ok) {
             covariance(cam, bp, scale[gs], quat[gs], G);
             float4 ra = *reinterpret_cast<const float4 *>(r);
@@ -507,85 +557,96 @@ __global__ void __launch_bounds__(256) k_project_bwd(
                 for (int i = 0; i < 4; ++i) dq[i] = (dqn[i] - G.qn[i] * dot) * G.qinv;
             }
         }
-        if (mask & UPS_GRAD_GAUSS) {
-            // the mean-scale term enters each set's scale gradient once
-            float sreg = vt.v[v].set_first ? scale_grad : 0.f;
-            float4 rc = *reinterpret_cast<const float4 *>(r + 8);  // dr dg db -
+        if (in && (mask & UPS_GRAD_GAUSS)) {
+            const float4 rc = *reinterpret_cast<const float4 *>(r + 8);  // dr dg db -
             if (direct) {
+                // over the zero fill, which holds the mean-scale term of the scales
                 d_mean_op[gs] = make_float4(dmu[0], dmu[1], dmu[2], dop);
-                d_scale[gs] = make_float4(ds[0] + sreg, ds[1] + sreg, ds[2] + sreg, 0.f);
+                d_scale[gs] = make_float4(ds[0] + scale_grad, ds[1] + scale_grad, ds[2] + scale_grad, 0.f);
                 d_quat[gs] = make_float4(dq[0], dq[1], dq[2], dq[3]);
                 d_color[gs] = make_float4(rc.x, rc.y, rc.z, 0.f);
                 // feature gradients as 16-byte moves (n_feat is a multiple of 4; the
                 // record's feature part starts 48 bytes into a 16-byte aligned record)
                 const float4 *rf = reinterpret_cast<const float4 *>(r + kG2Base);
-                float4 *df = reinterpret_cast<float4 *>(d_feat + (size_t)gs * n_feat);
+                float4 *df = reinterpret_cast<float4 *>(d_feat + gs * n_feat);
                 for (int c = 0; c < n_feat / 4; ++c) df[c] = rf[c];
-            } else {
-                float *dm = reinterpret_cast<float *>(d_mean_op + gs);
-                float *dsc = reinterpret_cast<float *>(d_scale + gs);
-                float *dqq = reinterpret_cast<float *>(d_quat + gs);
-                float *dc = reinterpret_cast<float *>(d_color + gs);
-                if (ok) {
-                    atomicAdd(dm + 0, dmu[0]);
-                    atomicAdd(dm + 1, dmu[1]);
-                    atomicAdd(dm + 2, dmu[2]);
-                    atomicAdd(dm + 3, dop);
-                    atomicAdd(dsc + 0, ds[0]);
-                    atomicAdd(dsc + 1, ds[1]);
-                    atomicAdd(dsc + 2, ds[2]);
-                    for (int i = 0; i < 4; ++i) atomicAdd(dqq + i, dq[i]);
-                    atomicAdd(dc + 0, rc.x);
-                    atomicAdd(dc + 1, rc.y);
-                    atomicAdd(dc + 2, rc.z);
-                    for (int c = 0; c < n_feat; ++c) atomicAdd(d_feat + (size_t)gs * n_feat + c, r[kG2Base + c]);
-                }
-                if (sreg != 0.f) {
-                    atomicAdd(dsc + 0, sreg);
-                    atomicAdd(dsc + 1, sreg);
-                    atomicAdd(dsc + 2, sreg);
-                }
+            } else if (ok) {
+                atomicAdd(d_mean_op + gs, make_float4(dmu[0], dmu[1], dmu[2], dop));
+                atomicAdd(d_scale + gs, make_float4(ds[0], ds[1], ds[2], 0.f));
+                atomicAdd(d_quat + gs, make_float4(dq[0], dq[1], dq[2], dq[3]));
+                atomicAdd(d_color + gs, make_float4(rc.x, rc.y, rc.z, 0.f));
+                for (int c = 0; c < n_feat; c += 4)
+                    atomicAdd(reinterpret_cast<float4 *>(d_feat + gs * n_feat + c),
+                              *reinterpret_cast<const float4 *>(r + kG2Base + c));
+            }
+        }
+        if (!(mask & UPS_GRAD_POSE)) continue;
+        // pose: a warp's Gaussian-views are mostly of one view
+        const int v0 = __shfl_sync(full, v, 0);
+        const bool same = __all_sync(full, !in || v == v0);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            float p = ok ? pose[i] : 0.f;
+            if (same) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(full, p, o);
+                if (lane == 0) atomicAdd(&s_pose[v0][i], p);
+            } else if (ok) {
+                atomicAdd(&s_pose[v][i], p);
             }
         }
     }
     if (!(mask & UPS_GRAD_POSE)) return;
-    // pose: one reduction per block when the block holds a single view, else
-    // per warp (or per lane when a warp straddles two views)
-    __shared__ float red[8][6];
-    __shared__ int vblock;
-    const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int v0 = __shfl_sync(full, v, 0);
-    bool wsame = __all_sync(full, v == v0);
-    if (!wsame) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            if (in && pose[i] != 0.f) atomicAdd(d_pose + 6 * v + i, pose[i]);
-            pose[i] = 0.f;
-        }
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) pose[i] += __shfl_xor_sync(full, pose[i], o);
-    if (threadIdx.x == 0) vblock = v;
     __syncthreads();
-    bool bsame = __syncthreads_and(v == vblock);
-    if (bsame) {
-        if (lane == 0)
-#pragma unroll
-            for (int i = 0; i < 6; ++i) red[w][i] = pose[i];
-        __syncthreads();
-        if (threadIdx.x < 6) {
-            float s = 0.f;
-            for (int ww = 0; ww < (int)(blockDim.x >> 5); ++ww) s += red[ww][threadIdx.x];
-            atomicAdd(d_pose + 6 * vblock + threadIdx.x, s);
-        }
-    } else if (lane == 0 && wsame) {
-#pragma unroll
-        for (int i = 0; i < 6; ++i) atomicAdd(d_pose + 6 * v0 + i, pose[i]);
+    for (int i = threadIdx.x; i < 6 * vt.n; i += kBwdThreads) {
+        const float p = (&s_pose[0][0])[i];
+        if (p != 0.f) atomicAdd(d_pose + i, p);
     }
 }
+
+// Zero gradients of the sets the views read, scale_grad in the scales (the
+// mean-scale term).  256 Gaussians a block, a view per grid row.
+__global__ void __launch_bounds__(256) k_zero_grads(ViewTable vt, int N, int n_feat, float scale_grad,
+                                                    float4 *__restrict__ d_mean_op, float4 *__restrict__ d_scale,
+                                                    float4 *__restrict__ d_quat, float4 *__restrict__ d_color,
+                                                    float *__restrict__ d_feat) {
+    const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+    const int g0 = blockIdx.x * 256, g = g0 + threadIdx.x;
+    const size_t base = (size_t)vt.v[blockIdx.y].set * N;
+    if (g < N) {
+        d_mean_op[base + g] = z;
+        d_scale[base + g] = make_float4(scale_grad, scale_grad, scale_grad, 0.f);
+        d_quat[base + g] = z;
+        d_color[base + g] = z;
+    }
+    float4 *f = reinterpret_cast<float4 *>(d_feat + (base + g0) * n_feat);
+    const int n = min(256, N - g0) * (n_feat / 4);
+    for (int i = threadIdx.x; i < n; i += 256) f[i] = z;
+}
+
+// dL/ds += scale_grad for every scale of n Gaussians (the sets that several
+// views read, whose gradients are accumulated)
+__global__ void __launch_bounds__(256) k_fill_scales(size_t n, float scale_grad, float4 *__restrict__ d_scale) {
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256)
+        d_scale[i] = make_float4(scale_grad, scale_grad, scale_grad, 0.f);
+}
+
+// Zeroes the records and bits of the listed Gaussian-views, a few percent of the
+// records, instead of a memset of all (0.9 GB at 8M Gaussian-views).
+__global__ void __launch_bounds__(256) k_clear_hits(HitList hits, float *__restrict__ g2, int stride) {
+    const int q = stride / 4;  // a thread 16 bytes
+    const size_t n = (size_t)*hits.count * q;
+    for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (size_t)gridDim.x * 256) {
+        const size_t h = i / q;
+        const int c = (int)(i - h * q);
+        const uint32_t gv = hits.list[h];
+        if (c == 0) hits.bits[gv >> 5] = 0u;  // every set bit of the word is listed
+        reinterpret_cast<float4 *>(g2 + (size_t)gv * stride)[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+}
+
+// CTAs of the grid-stride kernels over a hit list of up to n
+int hit_blocks(size_t n, int num_sms) { return (int)std::min<size_t>((n + 255) / 256, (size_t)num_sms * 4); }
 
 }  // namespace
 
@@ -633,11 +694,24 @@ cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaS
     return cudaGetLastError();
 }
 
-cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N, int per_view,
-                               int total, int n_feat, unsigned mask, float scale_grad,
-                               const ups_gaussians &g, const float *g2, const ups_gaussians *grad,
-                               float *d_pose, cudaStream_t st) {
-    if (total == 0) return cudaSuccess;
+cudaError_t launch_list_hits(const HitList &hits, size_t n_gv, cudaStream_t st) {
+    const size_t n_words = (n_gv + 31) / 32;
+    if (n_words == 0) return cudaSuccess;
+    k_list_hits<<<(unsigned)((n_words + 255) / 256), 256, 0, st>>>(hits, n_words);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clear_hits(const HitList &hits, size_t n_gv, float *g2, int n_feat, int num_sms, cudaStream_t st) {
+    if (n_gv == 0) return cudaSuccess;
+    k_clear_hits<<<hit_blocks(n_gv, num_sms), 256, 0, st>>>(hits, g2, g2_stride(n_feat));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N, int n_sets, int direct, int n_feat,
+                               unsigned mask, float scale_grad, const ups_gaussians &g, const float *g2,
+                               const HitList &hits, const ups_gaussians *grad, float *d_pose, int num_sms,
+                               cudaStream_t st) {
+    if (N == 0) return cudaSuccess;
     float4 *dm = nullptr, *ds = nullptr, *dq = nullptr, *dc = nullptr;
     float *df = nullptr;
     if (grad && (mask & UPS_GRAD_GAUSS)) {
@@ -646,11 +720,15 @@ cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N
         dq = reinterpret_cast<float4 *>(grad->quat);
         dc = reinterpret_cast<float4 *>(grad->color);
         df = grad->feat;
+        if (direct)
+            k_zero_grads<<<dim3((N + 255) / 256, vt.n), 256, 0, st>>>(vt, N, n_feat, scale_grad, dm, ds, dq, dc, df);
+        else if (scale_grad != 0.f)
+            k_fill_scales<<<num_sms * 4, 256, 0, st>>>((size_t)N * n_sets, scale_grad, ds);
     }
-    k_project_bwd<<<(total + 255) / 256, 256, 0, st>>>(
-        vt, bp, N, per_view, total, n_feat, mask, scale_grad,
-        reinterpret_cast<const float4 *>(g.mean_opacity), reinterpret_cast<const float4 *>(g.scale),
-        reinterpret_cast<const float4 *>(g.quat), g2, dm, ds, dq, dc, df, d_pose);
+    k_project_bwd<<<hit_blocks((size_t)N * vt.n, num_sms), kBwdThreads, 0, st>>>(
+        vt, bp, N, direct, n_feat, mask, scale_grad, reinterpret_cast<const float4 *>(g.mean_opacity),
+        reinterpret_cast<const float4 *>(g.scale), reinterpret_cast<const float4 *>(g.quat), g2, hits, dm, ds, dq, dc, df,
+        d_pose);
     return cudaGetLastError();
 }
 
