@@ -54,7 +54,7 @@ cudaError_t unc_view(int num_sms, cudaStream_t st, int W, int H, int nh, int pat
                      float *sigma, uint8_t *motion, float *scratch, int *launches);
 cudaError_t ssim_set_window();
 cudaError_t launch_ssim(const ViewTable &vt, const float *x, const float *y, const float *weight, float *G, float g,
-                        float *loss, float *dx, cudaStream_t st);
+                        float *loss, float *dx, int num_sms, cudaStream_t st);
 size_t lift_scratch_floats(size_t np_total);
 cudaError_t lift_all(int num_sms, cudaStream_t st, const ViewTable &vt, int nf, int nh, int patch, const float *feat,
                      const float *grid, const float *w1, const float *b1, const float *w2, const float *b2, float g,
@@ -853,7 +853,8 @@ ups_status ups_ssim_loss(ups_ctx *c, const float *color, const float *t_color, c
     stage_begin(c, "ssim", st);
     UPS_CUDA(c, cudaMemsetAsync(loss_dev, 0, sizeof(float), st));
     const float g = (float)((double)scale / (3.0 * (double)c->n_pix));
-    UPS_CUDA(c, launch_ssim(c->vt, color, t_color, weight, c->ssim_g.as<float>(), g, loss_dev, d_color, st));
+    UPS_CUDA(c, launch_ssim(c->vt, color, t_color, weight, c->ssim_g.as<float>(), g, loss_dev, d_color,
+                            c->num_sms, st));
     const int launches = d_color ? 2 : 1;
     stage_end(c, st, launches);
     return UPS_OK;
