@@ -143,9 +143,10 @@ cudaError_t keys_from_ranges(const uint2 *ranges, int nbins, uint32_t *keys, cud
 // in FP32 on the CUDA cores (op = transpose when ta / tb); column-major A
 // (m x k, or k x m when ta) and B (k x n, or n x k when tb).  Splits K over
 // several CTAs (atomic adds) when the output alone would not fill the GPU.
-// *launches (may be null) counts the kernels launched.
+// *launches (may be null) counts the kernels launched.  parts: sum K in parts of
+// at most 256 whatever m and n are (see gemm.cu).
 cudaError_t gemm_f32(cudaStream_t st, bool ta, bool tb, int m, int n, int k, float alpha, const float *A, int lda,
-                     const float *B, int ldb, float beta, float *C, int ldc, int num_sms, int *launches);
+                     const float *B, int ldb, float beta, float *C, int ldc, int num_sms, int *launches, bool parts = false);
 // Exclusive scan of n uint32 into uint64 (out has n+1 entries; out[n] = total).
 size_t scan_scratch_bytes(size_t n);
 cudaError_t exclusive_scan_u32_u64(const uint32_t *in, uint64_t *out, size_t n, void *scratch,

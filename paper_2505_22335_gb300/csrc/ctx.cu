@@ -47,11 +47,11 @@ cudaError_t anchor_update(const DevView &cam, const float *depth, const uint8_t 
                           float voxel, float margin, float near_z, long long capacity, float *opos, float *ofeat,
                           float *ooffsets, float *oscaling, float *olog, int *src_index, void *scratch,
                           uint64_t **summary_dev, cudaStream_t st, int *launches);
-size_t unc_scratch_floats(int max_patches);
-cudaError_t unc_view(int num_sms, cudaStream_t st, int W, int H, int nh, int patch, const float *grid, int wp,
-                     int hp, const float *R, const float *w1, const float *b1, const float *w2, const float *b2,
-                     float lambda, float g, float *loss, float *d_w1, float *d_b1, float *d_w2, float *d_b2,
-                     float *sigma, uint8_t *motion, float *scratch, int *launches);
+size_t unc_scratch_floats(size_t patches);
+cudaError_t unc_all(int num_sms, cudaStream_t st, const ViewTable &vt, int nh, int patch, const float *grid,
+                    const float *R, const float *w1, const float *b1, const float *w2, const float *b2, float lambda,
+                    float g, float *loss, float *d_w1, float *d_b1, float *d_w2, float *d_b2, float *sigma,
+                    uint8_t *motion, float *scratch, int *launches);
 cudaError_t ssim_set_window();
 cudaError_t launch_ssim(const ViewTable &vt, const float *x, const float *y, const float *weight, float *G, float g,
                         float *loss, float *dx, int num_sms, cudaStream_t st);
@@ -157,7 +157,7 @@ struct ups_ctx {
     bool capped = false;          // the last forward capped its tile lists
     DevBuf lift_scr;              // feature-lifting scratch of one view
     DevBuf ssim_g;                // D-SSIM window-term maps of all colour planes
-    DevBuf unc_scr;               // uncertainty-MLP patch scratch of one view
+    DevBuf unc_scr;               // uncertainty-MLP patch scratch of all views
     DevBuf anchor_scr;            // probabilistic-anchor update: flags, scans, voxel table
     uint64_t *h_anchor = nullptr;  // pinned: the anchor update's counts
     bool ssim_window = false;     // the SSIM window is in this device's constant memory
@@ -732,28 +732,20 @@ ups_status ups_uncertainty_mlp(ups_ctx *c, const ups_lift_cfg *lcfg, const float
     if (s != UPS_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c->last_stream = st;
-    int max_np = 0;
+    size_t patches = 0;
     for (int v = 0; v < c->vt.n; ++v) {
         const DevView &cam = c->vt.v[v];
-        max_np = std::max(max_np, ((cam.H + lcfg->patch - 1) / lcfg->patch) * ((cam.W + lcfg->patch - 1) / lcfg->patch));
+        patches += (size_t)((cam.H + lcfg->patch - 1) / lcfg->patch) * ((cam.W + lcfg->patch - 1) / lcfg->patch);
     }
-    UPS_CUDA(c, c->unc_scr.reserve(unc_scratch_floats(max_np) * sizeof(float)));
+    UPS_CUDA(c, c->unc_scr.reserve(unc_scratch_floats(patches) * sizeof(float)));
     stage_begin(c, "uncertainty_mlp", st);
     UPS_CUDA(c, cudaMemsetAsync(loss_dev, 0, sizeof(float), st));
     const float g = (float)((double)scale / (double)c->n_pix);
-    size_t grid_off = 0;
     int launches = 0;
-    for (int v = 0; v < c->vt.n; ++v) {
-        const DevView &cam = c->vt.v[v];
-        const int hp = (cam.H + lcfg->patch - 1) / lcfg->patch, wp = (cam.W + lcfg->patch - 1) / lcfg->patch;
-        const size_t P = (size_t)cam.pix_off;
-        UPS_CUDA(c, unc_view(c->num_sms, st, cam.W, cam.H, lcfg->n_h, lcfg->patch, dino + grid_off, wp, hp, R + P,
-                             mlp->w1, mlp->b1, mlp->w2, mlp->b2, lambda, g, loss_dev, d_mlp ? d_mlp->w1 : nullptr,
-                             d_mlp ? d_mlp->b1 : nullptr, d_mlp ? d_mlp->w2 : nullptr, d_mlp ? d_mlp->b2 : nullptr,
-                             sigma ? sigma + P : nullptr, motion ? motion + P : nullptr, c->unc_scr.as<float>(),
-                             &launches));
-        grid_off += (size_t)hp * wp * lcfg->n_h;
-    }
+    UPS_CUDA(c, unc_all(c->num_sms, st, c->vt, lcfg->n_h, lcfg->patch, dino, R, mlp->w1, mlp->b1, mlp->w2, mlp->b2, lambda,
+                        g, loss_dev, d_mlp ? d_mlp->w1 : nullptr, d_mlp ? d_mlp->b1 : nullptr,
+                        d_mlp ? d_mlp->w2 : nullptr, d_mlp ? d_mlp->b2 : nullptr, sigma, motion, c->unc_scr.as<float>(),
+                        &launches));
     stage_end(c, st, launches);
     return UPS_OK;
 }
