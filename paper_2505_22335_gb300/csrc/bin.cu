@@ -66,6 +66,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(ViewTable vt, float a
     const int tx = cam.tiles_x, ty = cam.tiles_y, ld = tx + 1, lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < ld * ty; i += kBinThreads) diff[i] = 0;
     __syncthreads();
+    const uint32_t top = (uint32_t)runs.N * (uint32_t)vt.n - 1u;  // an order that lost a wait may hold any id
     const int beg = runs.beg(blockIdx.x), end = runs.end(blockIdx.x);
     const uint32_t *sg = sorted_gv + (size_t)blockIdx.y * runs.N;
     constexpr int U = 4;  // gathers in flight per thread
@@ -73,7 +74,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(ViewTable vt, float a
         uint32_t gv[U];
         uint4 s[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) gv[u] = i0 + u * kBinThreads < end ? sg[i0 + u * kBinThreads] : 0xffffffffu;
+        for (int u = 0; u < U; ++u) gv[u] = i0 + u * kBinThreads < end ? min(sg[i0 + u * kBinThreads], top) : 0xffffffffu;
 #pragma unroll
         for (int u = 0; u < U; ++u) s[u] = gv[u] != 0xffffffffu ? span[gv[u]] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
@@ -323,6 +324,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
             }
         }
     }
+    const uint32_t top = (uint32_t)runs.N * (uint32_t)vt.n - 1u;
     const int beg = runs.beg(blockIdx.y), cnt = runs.end(blockIdx.y) - beg;
     const uint32_t *sg = sorted_gv + (size_t)blockIdx.x * runs.N + beg;
     // bits of word i of row r's live tiles inside columns [c0, c1]
@@ -356,7 +358,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int i = pos + u * kBinThreads + tid;
-                gv[u] = i < cnt ? sg[i] : 0xffffffffu;
+                gv[u] = i < cnt ? min(sg[i], top) : 0xffffffffu;
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {

@@ -115,9 +115,14 @@ size_t radix_hist_bytes(size_t n);
 cudaError_t radix_sort_u32(uint32_t **key_io, uint32_t **key_alt, uint32_t **val_io,
                            uint32_t **val_alt, size_t n, int end_bit, SortScratch &s,
                            cudaStream_t st);
-cudaError_t radix_sort_u64(uint64_t **key_io, uint64_t **key_alt, uint32_t **val_io,
-                           uint32_t **val_alt, size_t n, int end_bit, SortScratch &s,
-                           cudaStream_t st);
+// *sorted (val or val_alt) = the positions 0 .. n - 1 in ascending order of
+// their keys' bits [0, end_bit), stable; n < 2^31, end_bit <= 40; the keys are
+// overwritten.  *err is set (and ids may be missing or repeated) if a bounded
+// wait between CTAs ran out.  *launches: kernels launched.
+cudaError_t sorted_order_u32(uint32_t *key, uint32_t *key_alt, uint32_t *val, uint32_t *val_alt, size_t n, int end_bit,
+                             SortScratch &s, int num_sms, int *err, uint32_t **sorted, int *launches, cudaStream_t st);
+cudaError_t sorted_order_u64(uint64_t *key, uint64_t *key_alt, uint32_t *val, uint32_t *val_alt, size_t n, int end_bit,
+                             SortScratch &s, int num_sms, int *err, uint32_t **sorted, int *launches, cudaStream_t st);
 // Tile lists of the depth-ordered Gaussian-views (bin.cu): tile t of all
 // views keeps the first min(count, cap) Gaussian-views that meet it (cap =
 // kNoListCap: all), in depth order, at lists[ranges[t].x .. ranges[t].y); bit

@@ -141,7 +141,7 @@ struct ups_ctx {
     DevBuf cnt_sorted, off, scan_scr, ikey0, ikey1, ival0, ival1;
     DevBuf dec_scratch;  // decode backward: X, H, dL/dY, dL/dZ rows for the weight gradients
     SortScratch sort;
-    uint32_t *dval_sorted = nullptr, *ikey_sorted = nullptr, *ival_sorted = nullptr;
+    uint32_t *ikey_sorted = nullptr, *ival_sorted = nullptr;
     // device words of a forward and their pinned copy: the instance counters
     // and the list flag (cleared by every forward), the error flag
     struct Words {
@@ -583,13 +583,19 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     c->N = g->n;
     c->per_view = g->per_view ? 1 : 0;
     c->total_gv = total;
+    // (view, depth) order of the Gaussian-views: 32-bit keys (view in the top
+    // bits, depth bits above 0.125 m below) when the view index fits in 4 bits
+    // and the near plane is >= 0.125 m, else 64-bit keys
+    const int vbits = bits_for((size_t)n_views);
+    const bool k32 = vbits <= 4 && c->bp.near_z >= 0.125f;
+    const size_t key_bytes = k32 ? sizeof(uint32_t) : sizeof(uint64_t);
     // per-Gaussian-view scratch
     UPS_CUDA(c, c->xyzo.reserve(total * sizeof(float4)));
     UPS_CUDA(c, c->conic.reserve(total * sizeof(float4)));
     UPS_CUDA(c, c->rect.reserve(total * sizeof(uint2)));
     UPS_CUDA(c, c->count.reserve(total * sizeof(uint32_t)));
-    UPS_CUDA(c, c->dkey0.reserve(total * sizeof(uint64_t)));
-    UPS_CUDA(c, c->dkey1.reserve(total * sizeof(uint64_t)));
+    UPS_CUDA(c, c->dkey0.reserve(total * key_bytes));
+    UPS_CUDA(c, c->dkey1.reserve(total * key_bytes));
     UPS_CUDA(c, c->dval0.reserve(total * sizeof(uint32_t)));
     UPS_CUDA(c, c->dval1.reserve(total * sizeof(uint32_t)));
     UPS_CUDA(c, c->ranges.reserve((size_t)vt.total_tiles * sizeof(uint2)));
@@ -604,21 +610,15 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     }
     uint4 *span = rowwise ? c->span.as<uint4>() : nullptr, *more = rowwise ? c->more.as<uint4>() : nullptr;
 
-    // (view, depth) order of the Gaussian-views: 32-bit keys (view in the top
-    // bits, depth bits above 0.125 m below) when the view index fits in 4 bits
-    // and the near plane is >= 0.125 m, else 64-bit keys
-    int vbits = bits_for((size_t)n_views);
-    const bool k32 = vbits <= 4 && c->bp.near_z >= 0.125f;
-    uint32_t *dv = c->dval0.as<uint32_t>(), *dv_alt = c->dval1.as<uint32_t>();
     UPS_CUDA(c, cudaMemsetAsync(c->d_words, 0, offsetof(ups_ctx::Words, err), st));
     stage_begin(c, "project", st);
     if (k32)
         UPS_CUDA(c, launch_project_k32(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                                       c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint32_t>(), dv, vbits,
+                                       c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint32_t>(), nullptr, vbits,
                                        span, more, c->d_words->n_inst, st));
     else
         UPS_CUDA(c, launch_project(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                                   c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint64_t>(), dv, span, more,
+                                   c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint64_t>(), nullptr, span, more,
                                    c->d_words->n_inst, st));
     stage_end(c, st, 1);
     // the host needs the instance count to size the lists: its copy follows the
@@ -626,16 +626,17 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     UPS_CUDA(c, cudaMemcpyAsync(c->h_words, c->d_words, sizeof(ups_ctx::Words), cudaMemcpyDeviceToHost, st));
     UPS_CUDA(c, cudaEventRecord(c->words_ready, st));
     stage_begin(c, "depth_sort", st);
-    if (k32) {
-        uint32_t *dk = c->dkey0.as<uint32_t>(), *dk_alt = c->dkey1.as<uint32_t>();
-        UPS_CUDA(c, radix_sort_u32(&dk, &dk_alt, &dv, &dv_alt, total, 32, c->sort, st));
-        stage_end(c, st, radix_kernels(total, 32));
-    } else {
-        uint64_t *dk = c->dkey0.as<uint64_t>(), *dk_alt = c->dkey1.as<uint64_t>();
-        UPS_CUDA(c, radix_sort_u64(&dk, &dk_alt, &dv, &dv_alt, total, 32 + vbits, c->sort, st));
-        stage_end(c, st, radix_kernels(total, 32 + vbits));
-    }
-    c->dval_sorted = dv;
+    int sort_launches = 0;
+    uint32_t *dv = nullptr;
+    if (k32)
+        UPS_CUDA(c, sorted_order_u32(c->dkey0.as<uint32_t>(), c->dkey1.as<uint32_t>(), c->dval0.as<uint32_t>(),
+                                     c->dval1.as<uint32_t>(), total, 32, c->sort, c->num_sms, c->d_err, &dv,
+                                     &sort_launches, st));
+    else
+        UPS_CUDA(c, sorted_order_u64(c->dkey0.as<uint64_t>(), c->dkey1.as<uint64_t>(), c->dval0.as<uint32_t>(),
+                                     c->dval1.as<uint32_t>(), total, 32 + vbits, c->sort, c->num_sms, c->d_err, &dv,
+                                     &sort_launches, st));
+    stage_end(c, st, sort_launches);
     if (rowwise) {
         stage_begin(c, "tile_count", st);
         UPS_CUDA(c, bin_count(vt, c->bp.alpha_min, c->N, dv, span, more, c->xyzo.as<float4>(), c->conic.as<float4>(),

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kProjThreads) k_project(
             if (cnt) zf = min(__float_as_uint(z) - 0x3e000000u, zmask);
             dkey32[gv] = (vbits32 == 0 ? 0u : ((uint32_t)v << (32 - vbits32))) | zf;
         }
-        dval[gv] = (uint32_t)gv;
+        if (dval) dval[gv] = (uint32_t)gv;
     }
     if (!n_inst) return;
     // tile instances for the host's total: one atomic a block, spread over
@@ -265,7 +265,7 @@ __global__ void k_gather_counts(const uint32_t *__restrict__ sorted_gv,
                                 const uint32_t *__restrict__ count, uint32_t *__restrict__ out,
                                 int total) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < total) out[s] = count[sorted_gv[s]];
+    if (s < total) out[s] = count[min(sorted_gv[s], (uint32_t)total - 1u)];
 }
 
 // Instances of 32 consecutive depth-ordered Gaussian-views are written by one
@@ -295,7 +295,7 @@ __global__ void __launch_bounds__(256) k_emit(ViewTable vt, BlendParams bp, int 
     const uint64_t o = off[in ? s : total];
     const uint64_t o_end = off[min(s0 + 32, total)];
     const uint64_t o_beg = __shfl_sync(full, o, 0);
-    uint32_t gv = in ? sorted_gv[s] : 0u;
+    uint32_t gv = in ? min(sorted_gv[s], (uint32_t)total - 1u) : 0u;
     uint2 rc = make_uint2(0u, 0u);
     float4 xo = make_float4(0.f, 0.f, 0.f, 1.f), cn = make_float4(1.f, 0.f, 1.f, 0.f);
     const bool mine = in && off[s + 1] > o;
