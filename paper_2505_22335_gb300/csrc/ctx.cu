@@ -1015,11 +1015,11 @@ ups_status ups_decode_backward(ups_ctx *c, const ups_anchors *anc, const ups_mlp
     if ((s = set_device(c)) != UPS_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c->last_stream = st;
-    float *scratch = nullptr;
-    if ((mask & UPS_GRAD_MLP) && d_mlp) {
-        UPS_CUDA(c, c->dec_scratch.reserve(decode_bwd_scratch_bytes(anc->n, n_views, c->cfg.k, c->cfg.n_feat)));
-        scratch = c->dec_scratch.as<float>();
-    }
+    const size_t scratch_bytes = (mask & UPS_GRAD_MLP) && d_mlp
+                                     ? decode_bwd_scratch_bytes(anc->n, n_views, c->cfg.k, c->cfg.n_feat)
+                                     : ((size_t)anc->n * n_views + 4) * sizeof(uint32_t);
+    UPS_CUDA(c, c->dec_scratch.reserve(scratch_bytes));
+    float *scratch = c->dec_scratch.as<float>();
     const dbwd::StageHook hook{[](void *u, const char *name, bool begin, cudaStream_t s) {
                                    ups_ctx *cc = static_cast<ups_ctx *>(u);
                                    if (begin)

@@ -423,10 +423,10 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
     __syncthreads();
     const size_t NG = (size_t)a.A * a.K;
     float *sDX = sDXall + threadIdx.x;
-    for (int base = a.row_begin + blockIdx.x * dbwd::kRowsFp32; base < a.row_end;
-         base += gridDim.x * dbwd::kRowsFp32) {
-        const int row = base + threadIdx.x;
-        const bool valid = row < a.row_end;
+    const int end = a.rows ? (int)*a.n_rows : a.row_end;
+    for (int base = a.row_begin + blockIdx.x * dbwd::kRowsFp32; base < end; base += gridDim.x * dbwd::kRowsFp32) {
+        const bool valid = base + (int)threadIdx.x < end;
+        const int row = a.rows && valid ? (int)a.rows[base + threadIdx.x] : base + (int)threadIdx.x;
         const int an = valid ? row / V : 0, v = valid ? row - an * V : 0;
         const int lr = row - a.row_begin;
         const DevView &cam = vt.v[v];
@@ -455,6 +455,48 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
     dbwd::flush_pose(a, vt, aPose);
 }
 
+// Rows whose dL/dG is not all zero, for calls without MLP gradients.  A render
+// backward reaches a few percent of a large map's Gaussians (a tracking request
+// over 500k anchors: most rows are zero, and a zero row adds nothing), so one
+// read of dL/dG (128 B a Gaussian at 16 channels, the bound of this kernel)
+// saves the MLP backward of the others.  A warp a row, 32 rows one after another;
+// the row's arrays are read until one is not zero.
+constexpr int kLiveThreads = 256;
+__global__ void __launch_bounds__(kLiveThreads) k_live_rows(dbwd::Args a, int V, int n_rows, uint32_t *__restrict__ rows,
+                                                            uint32_t *__restrict__ n_live) {
+    __shared__ uint32_t s_bits[kLiveThreads / 32];
+    __shared__ uint32_t s_at;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int row0 = blockIdx.x * kLiveThreads + 32 * w;
+    const size_t NG = (size_t)a.A * a.K;
+    auto nonzero = [](float4 x) { return x.x != 0.f || x.y != 0.f || x.z != 0.f || x.w != 0.f; };  // NaN counts
+    uint32_t bits = 0;
+    for (int i = 0; i < 32 && row0 + i < n_rows; ++i) {
+        const int an = (row0 + i) / V, v = row0 + i - an * V;
+        const size_t g = (size_t)v * NG + (size_t)an * a.K;
+        bool hit = false;
+        if (lane < a.K)
+            hit = nonzero(a.d_mean_op[g + lane]) || nonzero(a.d_scale[g + lane]) || nonzero(a.d_quat[g + lane]) ||
+                  nonzero(a.d_color[g + lane]);
+        const float4 *f = reinterpret_cast<const float4 *>(a.d_feat + g * a.NF);
+        for (int k = lane; k < a.K * a.NF / 4 && !hit; k += 32) hit = nonzero(f[k]);
+        if (__any_sync(0xffffffffu, hit)) bits |= 1u << i;
+    }
+    if (lane == 0) s_bits[w] = bits;
+    __syncthreads();
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int i = 0; i < kLiveThreads / 32; ++i) {
+        const uint32_t c = __popc(s_bits[i]);
+        before += i < w ? c : 0u;
+        all += c;
+    }
+    if (all == 0) return;
+    if (threadIdx.x == 0) s_at = atomicAdd(n_live, all);
+    __syncthreads();
+    if (bits >> lane & 1u) rows[s_at + before + __popc(bits & ((1u << lane) - 1u))] = (uint32_t)(row0 + lane);
+}
+
 // shared memory of the backward rows kernel
 size_t bwd_rows_smem(int n_out) {
     return sizeof(float) * (kDin * 4 * kH + 4 * kH + n_out * kH + ((n_out + 3) & ~3) + kDX * dbwd::kRowsFp32);
@@ -465,6 +507,14 @@ size_t fwd_smem(int n_out) { return sizeof(float) * (kDin * 4 * kH + 4 * kH + n_
 }  // namespace
 
 size_t decode_bwd_rows_fp32_smem(int K, int NF) { return bwd_rows_smem(dbwd::n_out(K, NF)); }
+
+cudaError_t launch_live_rows(const dbwd::Args &a, int V, uint32_t *rows, uint32_t *n_rows, cudaStream_t st) {
+    cudaError_t e = cudaMemsetAsync(n_rows, 0, sizeof(uint32_t), st);
+    if (e != cudaSuccess) return e;
+    const int n = a.A * V;
+    k_live_rows<<<(n + kLiveThreads - 1) / kLiveThreads, kLiveThreads, 0, st>>>(a, V, n, rows, n_rows);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a, int num_sms, cudaStream_t st) {
     const size_t smem = bwd_rows_smem(dbwd::n_out(a.K, a.NF));

@@ -64,6 +64,10 @@ inline Scratch scratch_at(float *base, int ld, int n_out) {
 struct Args {
     int A, K, NF;
     int row_begin, row_end;  // rows of this launch (anchor-major)
+    // the launch's rows where only some have a nonzero dL/dG (null: all), and
+    // their number (device); without MLP gradients only
+    const uint32_t *rows;
+    const uint32_t *n_rows;
     const float *pos, *afeat, *offs, *ascale;
     const float *w1, *b1, *w2, *b2;
     const float4 *d_mean_op, *d_scale, *d_quat, *d_color;
@@ -216,6 +220,8 @@ struct StageHook {
 // per-row kernels (decode.cu: FP32 on the CUDA cores; decode_bwd_tc.cu: BF16
 // operands on the tensor cores) and the weight-gradient kernel
 cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a, int num_sms, cudaStream_t st);
+// rows (room for all) and *n_rows of the rows [0, A V) whose dL/dG is not all zero
+cudaError_t launch_live_rows(const dbwd::Args &a, int V, uint32_t *rows, uint32_t *n_rows, cudaStream_t st);
 cudaError_t launch_decode_bwd_rows_tc(const ViewTable &vt, const dbwd::Args &a, int num_sms, cudaStream_t st);
 size_t decode_bwd_rows_tc_smem(int NF, int K);
 // rows the per-row kernel's resident grid covers in one pass (FP32: 3 CTAs of

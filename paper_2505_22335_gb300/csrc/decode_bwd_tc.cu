@@ -714,7 +714,8 @@ cudaError_t launch_decode_bwd_rows_tc(const ViewTable &vt, const dbwd::Args &a, 
     return cudaGetLastError();
 }
 
-// Scratch bytes the decode backward needs (MLP gradients only).
+// Scratch bytes the decode backward needs for MLP gradients; without them it
+// needs (A V + 4) words for the list of rows.
 size_t decode_bwd_scratch_bytes(int A, int V, int K, int NF) {
     const int rows = std::min(A * V, kChunkRows);
     const int ld = (rows + 31) & ~31;
@@ -761,6 +762,18 @@ cudaError_t launch_decode_bwd(const ViewTable &vt, int A, int K, int NF, const u
     a.err = err;
     const bool want_mlp = (mask & UPS_GRAD_MLP) && d_mlp;
     const int rows = A * vt.n;
+    if (!want_mlp && !bf16) {
+        // one launch over the rows that have a gradient
+        uint32_t *list = reinterpret_cast<uint32_t *>(scratch);
+        a.rows = list + 4;
+        a.n_rows = list;
+        a.row_end = rows;
+        hook.fn(hook.user, "decode_bwd_rows", true, st);
+        cudaError_t e = launch_live_rows(a, vt.n, list + 4, list, st);
+        if (e == cudaSuccess) e = launch_decode_bwd_rows_fp32(vt, a, num_sms, st);
+        hook.fn(hook.user, "decode_bwd_rows", false, st);
+        return e;
+    }
     // chunks of whole passes of the per-row kernel's resident grid (a chunk of
     // 4.5 passes costs 5 on its slowest CTAs), at most kChunkRows rows
     const int wave = decode_bwd_rows_wave(bf16, K, NF, num_sms);
