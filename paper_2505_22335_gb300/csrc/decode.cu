@@ -13,6 +13,7 @@
 // and pre-activation gradients go to a feature-major scratch from which the
 // weight gradients are reduced by a separate kernel (decode_bwd_tc.cu).
 #include <algorithm>
+#include <initializer_list>
 
 #include "decode_bwd.cuh"
 
@@ -162,19 +163,91 @@ __device__ __forceinline__ void load_weights_T(const DecodeArgs &a, float *sW1T,
     for (int i = threadIdx.x; i < a.n_out; i += blockDim.x) sb2[i] = a.b2[i];
 }
 
-// forward decode: rows (threads) per CTA and resident CTAs per SM (its grid);
-// 2 x 384 (24 warps at 80 registers) measured 0.90 ms against 0.95 for 4 x 128
-// and 0.93 for 3 x 256 on the bench workload
-#ifndef UPS_DECF_THREADS
-#define UPS_DECF_THREADS 384
-#endif
-#ifndef UPS_DECF_CTAS
-#define UPS_DECF_CTAS 2
-#endif
-constexpr int kFwdThreads = UPS_DECF_THREADS, kFwdCtas = UPS_DECF_CTAS;
+// ---------------------------------------------------------------------------
+// forward
+// ---------------------------------------------------------------------------
+//
+// A warp takes 64 rows on its own, two a lane (rows lane and lane + 32), so that
+// every weight, a warp-uniform 16-byte shared load of two wavefronts, feeds both:
+// the kernel is bound by shared-memory and store wavefronts, then by the FMA
+// pipe.  The rows' inputs lie transposed in the warp's shared memory (one
+// wavefront an input and row group); the hidden values stay in registers.
+// Gaussians are stored two at a time as 32-byte records (full sectors) where K
+// is even and the outputs are 32-byte aligned.  Record of (row, k): row K + k.
+// Every element is rounded exactly as a scalar fmaf chain over the inputs in
+// order, and an output as four partial sums (s0 + s1) + (s2 + s3).
+// 800k rows (100k anchors x 10, 8 views, N_l 16): 0.67 ms; one row a lane 0.90
+// ms, a 4 x 4 register tile over lanes in rows and columns 0.81 ms (its 16-byte
+// loads take three to four wavefronts).
+constexpr int kFwdWarps = 16;  // warps per CTA at most (one CTA per SM)
+constexpr int kXT = 64;        // rows of a warp's XT [38][64]
 
-template <int NF>
-__global__ void __launch_bounds__(kFwdThreads, kFwdCtas) k_decode_fwd(ViewTable vt, DecodeArgs a,
+// W1_g x + b1_g of the lane's two rows (XT: at the lane's column), activated
+template <int ACT>
+__device__ __forceinline__ void hidden2(const float *sW1T, const float *sb1, int g, const float *XT, f2 (&h)[2][kH2]) {
+    const ulonglong2 *b = reinterpret_cast<const ulonglong2 *>(sb1 + g * kH);
+#pragma unroll
+    for (int q = 0; q < kH / 4; ++q) {
+        const ulonglong2 v = b[q];
+        h[0][2 * q] = h[1][2 * q] = v.x;
+        h[0][2 * q + 1] = h[1][2 * q + 1] = v.y;
+    }
+#pragma unroll 2
+    for (int k = 0; k < kDin; ++k) {
+        const float x0 = XT[k * kXT], x1 = XT[k * kXT + 32];
+        const f2 a = f2_make(x0, x0), c = f2_make(x1, x1);
+        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(sW1T + k * 4 * kH + g * kH);
+#pragma unroll
+        for (int q = 0; q < kH / 4; ++q) {
+            const ulonglong2 v = w[q];
+            h[0][2 * q] = f2_fma(v.x, a, h[0][2 * q]);
+            h[1][2 * q] = f2_fma(v.x, c, h[1][2 * q]);
+            h[0][2 * q + 1] = f2_fma(v.y, a, h[0][2 * q + 1]);
+            h[1][2 * q + 1] = f2_fma(v.y, c, h[1][2 * q + 1]);
+        }
+    }
+    activate<ACT>(h[0]);
+    activate<ACT>(h[1]);
+}
+
+// outputs r .. r + M - 1 of both rows
+template <int M>
+__device__ __forceinline__ void out2(const float *sW2, const float *sb2, int r, const f2 (&h)[2][kH2], float (&y)[2][M]) {
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        const ulonglong2 *w = reinterpret_cast<const ulonglong2 *>(sW2 + (r + j) * kH);
+        f2 a01[2], a23[2];
+        a01[0] = a01[1] = f2_make(sb2[r + j], 0.f);
+        a23[0] = a23[1] = 0ull;
+#pragma unroll
+        for (int q = 0; q < kH / 4; ++q) {
+            const ulonglong2 v = w[q];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                a01[i] = f2_fma(v.x, h[i][2 * q], a01[i]);
+                a23[i] = f2_fma(v.y, h[i][2 * q + 1], a23[i]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            float s0, s1, s2, s3;
+            f2_split(a01[i], s0, s1);
+            f2_split(a23[i], s2, s3);
+            y[i][j] = (s0 + s1) + (s2 + s3);
+        }
+    }
+}
+
+// 32 bytes at a 32-byte aligned address
+__device__ __forceinline__ void store8(float *p, float4 a, float4 b) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z),
+                 "f"(a.w), "f"(b.x), "f"(b.y), "f"(b.z), "f"(b.w)
+                 : "memory");
+}
+
+// PAIR: K is even and every output array 32-byte aligned
+template <int NF, bool PAIR>
+__global__ void __launch_bounds__(32 * kFwdWarps, 1) k_decode_fwd(ViewTable vt, DecodeArgs a, int split,
                                                     float4 *__restrict__ mean_op,
                                                     float4 *__restrict__ scale_out,
                                                     float4 *__restrict__ quat_out,
@@ -182,70 +255,126 @@ __global__ void __launch_bounds__(kFwdThreads, kFwdCtas) k_decode_fwd(ViewTable 
                                                     float *__restrict__ feat_out) {
     extern __shared__ float4 smem4[];
     float *sm = reinterpret_cast<float *>(smem4);
+    constexpr int P = PAIR ? 2 : 1;  // Gaussians a step
+    const int K = a.K, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     float *sW1T = sm, *sb1 = sW1T + kDin * 4 * kH, *sW2 = sb1 + 4 * kH, *sb2 = sW2 + a.n_out * kH;
+    float *XT = sb2 + ((a.n_out + 3) & ~3) + wid * (kDin * kXT) + lane;
     load_weights_T(a, sW1T, sb1, sW2, sb2);
     __syncthreads();
-    const int K = a.K;
-    const int rows = a.A * vt.n;
-    const size_t NG = (size_t)a.A * K;
-    for (int row = blockIdx.x * blockDim.x + threadIdx.x; row < rows; row += gridDim.x * blockDim.x) {
-        const int v = row / a.A, an = row - v * a.A;
-        const DevView &cam = vt.v[v];
-        float xt[6];
-        {
+    const int rows = a.A * vt.n, nw = blockDim.x >> 5;
+    const int tiles = (rows + kXT - 1) / kXT;
+    // Work items: a tile, or (split) one MLP of a tile, the costliest MLP first:
+    // features, covariance, colour, opacity.  They go round the SMs before the
+    // warps, so that a last, partial round loads every SM alike.
+    constexpr int kMlps = NF > 0 ? 4 : 3;
+    const int items = split ? kMlps * tiles : tiles;
+    for (int it = blockIdx.x + gridDim.x * wid; it < items; it += gridDim.x * nw) {
+        const int tile = it % tiles, first = (split ? it / tiles : 0) + (4 - kMlps), last = split ? first : 3;
+        int row[2], an[2];
+        bool on[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            row[i] = tile * kXT + 32 * i + lane;
+            on[i] = row[i] < rows;
+            row[i] = min(row[i], rows - 1);
+            const int v = row[i] / a.A;
+            an[i] = row[i] - v * a.A;
             float x[kDinP], delta[3], dist;
-            mlp_input(a, cam, an, x, delta, dist);
+            mlp_input(a, vt.v[v], an[i], x, delta, dist);
 #pragma unroll
-            for (int u = 0; u < 6; ++u) xt[u] = x[kFin + u];
+            for (int k = 0; k < kDin; ++k) XT[k * kXT + 32 * i] = x[k];  // read back by this lane only
         }
-        const float *af = a.afeat + (size_t)an * kFin;
-        f2 z[kH2];
-        const size_t gbase = (size_t)v * NG + (size_t)an * K;
-        // opacity, and the mean
-        hidden_T(sW1T, sb1, 0, af, xt, z);
-        activate<0>(z);
-        const float px = a.pos[3 * an], py = a.pos[3 * an + 1], pz = a.pos[3 * an + 2];
+        // the P records from k of row i
+        auto put = [&](float4 *base, int i, int k, const float4 (&v)[P]) {
+            if (!on[i]) return;
+            float4 *p = base + (size_t)row[i] * K + k;
+            if constexpr (PAIR)
+                store8(reinterpret_cast<float *>(p), v[0], v[P - 1]);
+            else
+                *p = v[0];
+        };
 #pragma unroll 1
-        for (int k = 0; k < K; ++k) {
-            const float *o3 = a.offs + ((size_t)an * K + k) * 3;
-            mean_op[gbase + k] = make_float4(px + o3[0], py + o3[1], pz + o3[2],
-                                             opacity_act(out_row(sW2, sb2, k, z), a.op_tanh));
-        }
-        // covariance: 3 scale + 4 quaternion per Gaussian
-        hidden_T(sW1T, sb1, 1, af, xt, z);
-        activate<0>(z);
-        const float lx = a.ascale[3 * an], ly = a.ascale[3 * an + 1], lz = a.ascale[3 * an + 2];
+        for (int order = first; order <= last; ++order) {
+            f2 h[2][kH2];
+            if (order == 3) {  // opacity, and the mean
+                hidden2<0>(sW1T, sb1, 0, XT, h);
 #pragma unroll 1
-        for (int k = 0; k < K; ++k) {
-            const int r = K + 7 * k;
-            const float s0 = lx * sigm(out_row(sW2, sb2, r, z));
-            const float s1 = ly * sigm(out_row(sW2, sb2, r + 1, z));
-            const float s2 = lz * sigm(out_row(sW2, sb2, r + 2, z));
-            const float q0 = out_row(sW2, sb2, r + 3, z), q1 = out_row(sW2, sb2, r + 4, z);
-            const float q2 = out_row(sW2, sb2, r + 5, z), q3 = out_row(sW2, sb2, r + 6, z);
-            scale_out[gbase + k] = make_float4(s0, s1, s2, 0.f);
-            quat_out[gbase + k] = make_float4(q0, q1, q2, q3);
-        }
-        // colour
-        hidden_T(sW1T, sb1, 2, af, xt, z);
-        activate<0>(z);
-#pragma unroll 1
-        for (int k = 0; k < K; ++k) {
-            const int r = 8 * K + 3 * k;
-            color_out[gbase + k] = make_float4(sigm(out_row(sW2, sb2, r, z)), sigm(out_row(sW2, sb2, r + 1, z)),
-                                               sigm(out_row(sW2, sb2, r + 2, z)), 0.f);
-        }
-        if (NF > 0) {
-            hidden_T(sW1T, sb1, 3, af, xt, z);
-            activate<1>(z);
-#pragma unroll 1
-            for (int k = 0; k < K; ++k) {
-                float4 *dst = reinterpret_cast<float4 *>(feat_out + (gbase + k) * NF);
-                const int r = 11 * K + NF * k;
+                for (int k = 0; k < K; k += P) {
+                    float y[2][P];
+                    out2<P>(sW2, sb2, k, h, y);
 #pragma unroll
-                for (int c = 0; c < NF / 4; ++c)
-                    dst[c] = make_float4(out_row(sW2, sb2, r + 4 * c, z), out_row(sW2, sb2, r + 4 * c + 1, z),
-                                         out_row(sW2, sb2, r + 4 * c + 2, z), out_row(sW2, sb2, r + 4 * c + 3, z));
+                    for (int i = 0; i < 2; ++i) {
+                        const float *p = a.pos + 3 * an[i], *o3 = a.offs + ((size_t)an[i] * K + k) * 3;
+                        float4 m[P];
+#pragma unroll
+                        for (int j = 0; j < P; ++j)
+                            m[j] = make_float4(p[0] + o3[3 * j], p[1] + o3[3 * j + 1], p[2] + o3[3 * j + 2],
+                                               opacity_act(y[i][j], a.op_tanh));
+                        put(mean_op, i, k, m);
+                    }
+                }
+            } else if (order == 1) {  // covariance: 3 scale + 4 quaternion per Gaussian
+                hidden2<0>(sW1T, sb1, 1, XT, h);
+#pragma unroll 1
+                for (int k = 0; k < K; k += P) {
+                    float4 s[2][P];
+#pragma unroll
+                    for (int j = 0; j < P; ++j) {
+                        float y[2][3];
+                        out2<3>(sW2, sb2, K + 7 * (k + j), h, y);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const float *l = a.ascale + 3 * an[i];
+                            s[i][j] = make_float4(l[0] * sigm(y[i][0]), l[1] * sigm(y[i][1]), l[2] * sigm(y[i][2]), 0.f);
+                        }
+                    }
+                    put(scale_out, 0, k, s[0]);
+                    put(scale_out, 1, k, s[1]);
+#pragma unroll
+                    for (int j = 0; j < P; ++j) {
+                        float y[2][4];
+                        out2<4>(sW2, sb2, K + 7 * (k + j) + 3, h, y);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) s[i][j] = make_float4(y[i][0], y[i][1], y[i][2], y[i][3]);
+                    }
+                    put(quat_out, 0, k, s[0]);
+                    put(quat_out, 1, k, s[1]);
+                }
+            } else if (order == 2) {  // colour
+                hidden2<0>(sW1T, sb1, 2, XT, h);
+#pragma unroll 1
+                for (int k = 0; k < K; k += P) {
+                    float4 c[2][P];
+#pragma unroll
+                    for (int j = 0; j < P; ++j) {
+                        float y[2][3];
+                        out2<3>(sW2, sb2, 8 * K + 3 * (k + j), h, y);
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) c[i][j] = make_float4(sigm(y[i][0]), sigm(y[i][1]), sigm(y[i][2]), 0.f);
+                    }
+                    put(color_out, 0, k, c[0]);
+                    put(color_out, 1, k, c[1]);
+                }
+            } else if (NF > 0) {
+                hidden2<1>(sW1T, sb1, 3, XT, h);
+#pragma unroll 1
+                for (int f = 0; f < K * NF; f += 8) {
+                    float y[2][8];
+                    out2<8>(sW2, sb2, 11 * K + f, h, y);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (!on[i]) continue;
+                        float *p = feat_out + (size_t)row[i] * K * NF + f;
+                        const float4 lo = make_float4(y[i][0], y[i][1], y[i][2], y[i][3]);
+                        const float4 hi = make_float4(y[i][4], y[i][5], y[i][6], y[i][7]);
+                        if constexpr (PAIR) {
+                            store8(p, lo, hi);
+                        } else {
+                            reinterpret_cast<float4 *>(p)[0] = lo;
+                            reinterpret_cast<float4 *>(p)[1] = hi;
+                        }
+                    }
+                }
             }
         }
     }
@@ -502,7 +631,10 @@ size_t bwd_rows_smem(int n_out) {
     return sizeof(float) * (kDin * 4 * kH + 4 * kH + n_out * kH + ((n_out + 3) & ~3) + kDX * dbwd::kRowsFp32);
 }
 
-size_t fwd_smem(int n_out) { return sizeof(float) * (kDin * 4 * kH + 4 * kH + n_out * kH + n_out); }
+size_t fwd_smem(int n_out, int warps) {
+    return sizeof(float) * (kDin * 4 * kH + 4 * kH + (size_t)n_out * kH + ((n_out + 3) & ~3) +
+                            (size_t)warps * kDin * kXT);
+}
 
 }  // namespace
 
@@ -543,18 +675,39 @@ cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const u
                               cudaStream_t st) {
     DecodeArgs a{A, K, NF, K * (11 + NF), anc.pos, anc.feat, anc.offsets, anc.scaling,
                  mlp.w1, mlp.b1, mlp.w2, mlp.b2, op_tanh};
-    size_t smem = fwd_smem(a.n_out);
+    // as many warps as the weights leave room for (16 at 270 outputs, 15 at 430)
+    int warps = kFwdWarps;
+    while (warps > 1 && fwd_smem(a.n_out, warps) > kMaxSmem) --warps;
+    // one CTA per SM.  Fewer than four rounds of tiles are split by MLP: 10k rows
+    // 45 us (77 in tiles), 184k rows 191 (197); with more, sharing a tile's inputs
+    // is worth more than even rounds (800k rows 675 against 721).  Eight warps at
+    // least, to load the weights.
+    const int tiles = (A * vt.n + kXT - 1) / kXT;
+    const int split = tiles < 4 * num_sms * warps;
+    const int items = split ? tiles * (NF > 0 ? 4 : 3) : tiles;
+    warps = std::min(warps, std::max(8, (items + num_sms - 1) / num_sms));
+    const size_t smem = fwd_smem(a.n_out, warps);
     if (smem > kMaxSmem) return cudaErrorInvalidConfiguration;
-    int rows = A * vt.n;
-    int blocks = std::max(1, std::min((rows + kFwdThreads - 1) / kFwdThreads, num_sms * kFwdCtas));
-#define UPS_DEC(NFV)                                                                        \
-    do {                                                                                    \
-        cudaFuncSetAttribute(k_decode_fwd<NFV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem);                                                    \
-        k_decode_fwd<NFV><<<blocks, kFwdThreads, smem, st>>>(                               \
-            vt, a, reinterpret_cast<float4 *>(out.mean_opacity),                            \
-            reinterpret_cast<float4 *>(out.scale), reinterpret_cast<float4 *>(out.quat),    \
-            reinterpret_cast<float4 *>(out.color), out.feat);                               \
+    const int blocks = std::max(1, std::min(items, num_sms));
+    bool pair = K % 2 == 0;
+    for (const void *p : {(const void *)out.mean_opacity, (const void *)out.scale, (const void *)out.quat,
+                          (const void *)out.color, (const void *)out.feat})
+        pair = pair && reinterpret_cast<uintptr_t>(p) % 32 == 0;
+#define UPS_DEC1(NFV, PAIRV)                                                                       \
+    do {                                                                                           \
+        cudaFuncSetAttribute(k_decode_fwd<NFV, PAIRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                             (int)smem);                                                           \
+        k_decode_fwd<NFV, PAIRV><<<blocks, 32 * warps, smem, st>>>(                                \
+            vt, a, split, reinterpret_cast<float4 *>(out.mean_opacity),                            \
+            reinterpret_cast<float4 *>(out.scale), reinterpret_cast<float4 *>(out.quat),           \
+            reinterpret_cast<float4 *>(out.color), out.feat);                                      \
+    } while (0)
+#define UPS_DEC(NFV)              \
+    do {                          \
+        if (pair)                 \
+            UPS_DEC1(NFV, true);  \
+        else                      \
+            UPS_DEC1(NFV, false); \
     } while (0)
     switch (NF) {
         case 0: UPS_DEC(0); break;
@@ -563,6 +716,7 @@ cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const u
         default: return cudaErrorInvalidValue;
     }
 #undef UPS_DEC
+#undef UPS_DEC1
     return cudaGetLastError();
 }
 
