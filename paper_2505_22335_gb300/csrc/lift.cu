@@ -528,17 +528,27 @@ __global__ void __launch_bounds__(kFT, 1) k_lift_fused(
 //   TMEM columns [64, 80): dW1, accumulated over all of the CTA's chunks
 //   TMEM columns [128, 256): the Gram, likewise
 //   TMEM columns [256, 384): M hi, lo; [384, 448): H hi, lo; [448, 512): dZ hi, lo (A operands)
-// Thread 0 issues the Z and M H MMAs (`mh_bar` completes each), thread kGramTid
-// the Gram and dW1 MMAs (`g_bar` completes them, waited at the next chunk).  A
-// warp reads TMEM lanes 32 (w % 4) .. + 31, so thread (warp w, lane i) owns
-// hidden unit j = 32 (w % 4) + i and the chunk's pixels 32 (w / 4) .. + 31 from
-// Z on, keeping H of them in registers; per-pixel sums over hidden units are
-// reduce-scattered over the warp's lanes and added over the four warps of a
-// pixel half.  H reaches M H's B operand in the MN-major layout straight from
-// the registers; a chunk's global inputs arrive by cp.async a chunk ahead.
+// 16 worker warps, and one that issues all MMAs (`mh_bar` completes Z and M H,
+// `g_bar` the Gram and dW1, waited at the next chunk): a chunk's 24 M H or 24 Gram
+// and dW1 MMAs hold their issuer for 1100 to 1800 cycles, which a worker spent at
+// the others' expense.  A warp reads TMEM lanes 32 (w % 4) .. + 31, so thread
+// (warp w, lane i) owns hidden unit j = 32 (w % 4) + i and the chunk's pixels
+// 16 (w / 4) .. + 15 from Z on, keeping H of them in registers; per-pixel sums over
+// hidden units are reduce-scattered over the warp's lanes and added over the four
+// warps of a pixel group, each of which then does the group's per-pixel terms for
+// itself (five barriers a chunk).  A cell's last chunk runs in steps of 16 pixels
+// (196 pixels at 14-pixel patches: 3 chunks of 64 and one step).  H reaches M H's B
+// operand in the MN-major layout straight from the registers; a chunk's global
+// inputs arrive by cp.async a chunk ahead.
+// 8 x 640x480 at n_h = 384: 2.57 ms, 2.82 with 8 warps, MMAs issued by workers and
+// eleven barriers.  What bounds it are the phases' latencies, one after another
+// (clock64 over a chunk of about 13k cycles: M H 2.6k, dF~ 2.3k, dZ 2.0k, Z 1.5k,
+// the cosine terms 0.9k).
 namespace lt {
 constexpr int kP = 64;       // pixels per chunk
-constexpr int kT = 256;      // threads
+constexpr int kT = 512;      // worker threads
+constexpr int kAll = kT + 32;  // and the warp that issues the MMAs
+constexpr int kIssueWarp = kT / 32;
 constexpr int kHS = kP + 4;  // row stride of the FP32 hidden-major arrays
 // TMEM columns; the A operands (M, and H as the Gram's A) sit in TMEM as BF16
 // pairs (row = lane), so the MMAs read only their B operands from shared memory
@@ -551,7 +561,6 @@ constexpr int oHBhi = 0, oHBlo = 16384;        // H [128 k][64 p] (B of M H)
 constexpr int oBHhi = 32768, oBHlo = 49152;    // b H [128 i][64 p] (B of the Gram)
 constexpr int kOpBytes = 65536;
 constexpr int kWait = 1 << 22;
-constexpr int kGramTid = 128;  // issues the Gram and dW1 MMAs
 // M H's B operand H (K = 128 hidden units x N = 64 pixels) in the MN-major layout
 // without swizzle: core matrices of 8 hidden rows x 8 pixels (16 bytes per row, 128
 // bytes each), 8 along N then 16 along K, so that a thread writes its hidden unit's
@@ -583,14 +592,13 @@ struct LiftTcSmem {  // after the operand tiles (1 KB aligned); the arrays read 
     float Fc[2][16][lt::kHS];        // F~ of the chunk, channel-major
     float dF0[2][16][lt::kP];        // dL/dF~ accumulated before this call, channel-major
     float w4[lt::kP][4];             // bilinear weights of the chunk's pixels
-    float ab[lt::kP][2];             // a_p, b_p
-    float aw[lt::kP][4];             // a_p w_k(p)
-    float Dpart[4][kLiftHidden];
+    float ab[lt::kT / 32][16][8];    // per warp and pixel of its group: a_p w_k(p), b_p
+    float Dpart[4][4][kLiftHidden];  // the cell's D per pixel group (one thread a value), corner and unit
     float red[4][lt::kP][2];         // partial H.e, H.(M H + 2 u) per 32 hidden units
     uint32_t FcT[2][512];            // F~ as BF16 hi / lo, K-major [16 channels][64 pixels] (B of dW1)
     float wpx[2][lt::kP];            // loss weights of the chunk's pixels
     float sS[2][4], sG[2][12];       // s of the corners, the cell's corner Gram (10 used)
-    int pix[lt::kP];                 // pixel index in the view, -1: none
+    int pix[2][lt::kP];              // pixel index in the view (by chunk parity), -1: none
     int vwp[UPS_MAX_VIEWS], vhp[UPS_MAX_VIEWS], vbase[UPS_MAX_VIEWS];  // each view's patch grid, first cell
     uint64_t mh_bar, g_bar;
     uint32_t tmem_base;
@@ -601,7 +609,7 @@ static_assert(offsetof(LiftTcSmem, Hh) == 0 && offsetof(LiftTcSmem, W1A) % 16 ==
                   offsetof(LiftTcSmem, W1r) % 16 == 0 && offsetof(LiftTcSmem, FcT) % 16 == 0 &&
                   offsetof(LiftTcSmem, E) % 16 == 0 && offsetof(LiftTcSmem, Fc) % 16 == 0 &&
                   offsetof(LiftTcSmem, dF0) % 16 == 0 &&
-                  offsetof(LiftTcSmem, w4) % 16 == 0 && offsetof(LiftTcSmem, ab) % 8 == 0 &&
+                  offsetof(LiftTcSmem, w4) % 16 == 0 && offsetof(LiftTcSmem, ab) % 16 == 0 &&
                   offsetof(LiftTcSmem, mh_bar) % 8 == 0,
               "vector, bulk-copy and mbarrier alignment of the lifting kernel's shared arrays");
 
@@ -610,6 +618,7 @@ static_assert(offsetof(LiftTcSmem, Hh) == 0 && offsetof(LiftTcSmem, W1A) % 16 ==
 // table in shared memory (the same numbering as cell_view).
 struct CellGeo {
     int v, W, wp, hp, base, x0, y0, xs, ys, nx, npx;
+    float inv_nx;
     size_t HW, P;
 };
 __device__ __forceinline__ CellGeo cell_geo(const LiftTcSmem &S, const ViewTable &vt, int patch, int cell) {
@@ -634,7 +643,14 @@ __device__ __forceinline__ CellGeo cell_geo(const LiftTcSmem &S, const ViewTable
     const int ye = g.y0 + 1 >= cv.hp ? H : min(H, cell_start(g.y0 + 1, patch));
     g.nx = max(0, xe - g.xs);
     g.npx = g.nx * max(0, ye - g.ys);
+    g.inv_nx = 1.f / (float)max(g.nx, 1);
     return g;
+}
+// image row of the cell's pixel q, counted from its first: q / nx.  In FP32 with
+// half a pixel added the quotient is off by less than 1e-6 of itself, and at
+// least 0.5 / nx from a whole number: exact for cells of up to 2^18 pixels.
+__device__ __forceinline__ int cell_row(const CellGeo &g, int q) {
+    return g.npx <= (1 << 18) ? (int)(((float)q + 0.5f) * g.inv_nx) : q / g.nx;
 }
 // corner k of the cell (bit 0: next column, bit 1: next row, clamped to the grid)
 __device__ __forceinline__ int cell_corner(const CellGeo &g, int k) {
@@ -659,29 +675,30 @@ __device__ __forceinline__ void cp_async_wait() {
 }
 
 // Issues the copies of chunk (cell, q0)'s global inputs into buffer B (all
-// kT threads call it): F~ and dL/dF~ accumulated before the call (thread t:
-// pixel t % kP, channels t / kP + 4 r), the loss weights (t < kP), and the
-// cell's corner rows of E, s and its Gram.  Pixels past the cell's end read
-// nothing and hold 0.
-__device__ __forceinline__ void lift_chunk_issue(LiftTcSmem &S, int B, const ViewTable &vt, int patch, int cell,
-                                                 int q0, const float *__restrict__ feat_all,
+// kT threads call it): F~ (thread t < 256: pixel t % kP, channels 4 (t / kP) +
+// [0, 4), which the same thread turns into the TF32 operand), dL/dF~
+// accumulated before the call (the other threads, the same split), the loss
+// weights (t < kP), and the cell's corner rows of E, s and its Gram.  Pixels
+// past the cell's end read nothing and hold 0.
+__device__ __forceinline__ void lift_chunk_issue(LiftTcSmem &S, int B, const CellGeo &g, int cell, int q0, const float *__restrict__ feat_all,
                                                  const float *__restrict__ d_feat_all,
                                                  const float *__restrict__ weight_all, const float *__restrict__ E,
                                                  const float *__restrict__ s, const float *__restrict__ gram, int tid) {
     using namespace lt;
-    const CellGeo g = cell_geo(S, vt, patch, cell);
+    static_assert(kT == 8 * kP, "four channels a thread, F~ and dL/dF~");
     {
-        const int p = tid & (kP - 1), q = q0 + p;
+        const int p = tid & (kP - 1), q = q0 + p, c0 = 4 * ((tid / kP) & 3);
         const bool in = q < g.npx;
-        const int yq = in ? q / g.nx : 0;
+        const int yq = in ? cell_row(g, q) : 0;
         const size_t pidx = in ? (size_t)(g.ys + yq) * g.W + g.xs + (q - yq * g.nx) : 0;
-        const float *feat = feat_all + (size_t)16 * g.P;
-        const float *df = d_feat_all ? d_feat_all + (size_t)16 * g.P : nullptr;
+        if (tid < 4 * kP) {
+            const float *feat = feat_all + (size_t)16 * g.P;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int c = (tid / kP) + 4 * r;
-            cp_async4(&S.Fc[B][c][p], feat + (size_t)c * g.HW + pidx, in);
-            if (df) cp_async4(&S.dF0[B][c][p], df + (size_t)c * g.HW + pidx, in);
+            for (int c = c0; c < c0 + 4; ++c) cp_async4(&S.Fc[B][c][p], feat + (size_t)c * g.HW + pidx, in);
+        } else if (d_feat_all) {
+            const float *df = d_feat_all + (size_t)16 * g.P;
+#pragma unroll
+            for (int c = c0; c < c0 + 4; ++c) cp_async4(&S.dF0[B][c][p], df + (size_t)c * g.HW + pidx, in);
         }
         if (weight_all && tid < kP) cp_async4(&S.wpx[B][p], weight_all + g.P + pidx, in);
     }
@@ -733,11 +750,11 @@ __device__ __forceinline__ void put8_split(unsigned char *hi, unsigned char *lo,
     *reinterpret_cast<uint4 *>(lo + off) = l;
 }
 
-// Sum over the warp's lanes of v[lane]: the 32 values of every lane are
-// reduce-scattered, lane l keeps the total of entry l.
-__device__ __forceinline__ float warp_rs32(float (&v)[32], int lane) {
+// Sums over the warp's lanes of each of a lane's 16 values, reduce-scattered:
+// lanes l and l + 16 return the total of value l % 16.
+__device__ __forceinline__ float warp_rs16(float (&v)[16], int lane) {
 #pragma unroll
-    for (int s = 16; s >= 1; s >>= 1) {
+    for (int s = 8; s >= 1; s >>= 1) {
         const bool up = (lane & s) != 0;
 #pragma unroll
         for (int t = 0; t < s; ++t) {
@@ -746,10 +763,10 @@ __device__ __forceinline__ float warp_rs32(float (&v)[32], int lane) {
             v[t] = keep + __shfl_xor_sync(0xffffffffu, send, s);
         }
     }
-    return v[0];
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 16);
 }
 
-__global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
+__global__ void __launch_bounds__(lt::kAll, 1) k_lift_tc(
     ViewTable vt, int n_cells, int patch, const float *__restrict__ feat_all, const float *__restrict__ w1,
     const float *__restrict__ b1, const float *__restrict__ Mg, const float *__restrict__ E,
     const float *__restrict__ s, const float *__restrict__ u, const float *__restrict__ beta,
@@ -764,6 +781,7 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
     LiftTcSmem &S = *reinterpret_cast<LiftTcSmem *>(op + kOpBytes);
     const uint32_t sop = umma::smem_addr(op);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int warp_u = __shfl_sync(0xffffffffu, warp, 0);  // the same, known to be uniform
     for (int i = tid; i < kLiftHidden * NF; i += kT) {
         const int j = i / NF, c = i - j * NF;
         S.W1r[j][c] = w1[i];
@@ -797,12 +815,13 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
     __syncthreads();
     umma::fence_after();
     const uint32_t tmem = S.tmem_base;
-    const int jt = 32 * (warp & 3) + lane, ph = 32 * (warp >> 2);
+    const int jt = 32 * (warp & 3) + lane, ph = 16 * (warp >> 2);
     const uint32_t lane_addr = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
     // M (symmetric) as BF16 hi/lo pairs into TMEM: lane jt = row jt, the
-    // thread's warp half writes k in [64 (w / 4), + 64)
-#pragma unroll 1
-    for (int k0 = 2 * ph; k0 < 2 * ph + 64; k0 += 32) {
+    // thread's warp quarter writes k in [32 (w / 4), + 32)
+    const bool worker = warp_u < kIssueWarp;
+    if (worker) {
+        const int k0 = 2 * ph;
         uint32_t hi[16], lo[16];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -823,13 +842,17 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
     float t_loss = 0.f, t_sb = 0.f;
     uint32_t mh_phase = 0, g_phase = 0;
     bool g_pending = false, g_started = false, mh_pending = false, ok = true;
-    const uint32_t id_mh = umma::idesc(umma::kBF16, 128, kP), id_g = umma::idesc(umma::kBF16, 128, 128),
-                   id_dw = umma::idesc(umma::kBF16, 128, NF), id_z = umma::idesc(umma::kTF32, 128, kP);
+    const uint32_t id_mh = umma::idesc(umma::kBF16, 128, 0), id_g = umma::idesc(umma::kBF16, 128, 128),
+                   id_dw = umma::idesc(umma::kBF16, 128, NF), id_z = umma::idesc(umma::kTF32, 128, 0);
+    // (N of M H and Z is the chunk's, in steps of 16 pixels)
     float *red = &S.red[0][0][0];  // [4][kP][2]
+    if (worker)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) S.Dpart[warp >> 2][k][jt] = 0.f;
     // the chunk whose inputs are in flight to buffer buf (cell -1: none)
     int pre_cell = -1, pre_q0 = 0, buf = 0;
-    if ((int)blockIdx.x < n_cells) {
-        lift_chunk_issue(S, 0, vt, patch, blockIdx.x, 0, feat_all, d_feat_all, weight_all, E, s, gram, tid);
+    if (worker && (int)blockIdx.x < n_cells) {
+        lift_chunk_issue(S, 0, cell_geo(S, vt, patch, blockIdx.x), blockIdx.x, 0, feat_all, d_feat_all, weight_all, E, s, gram, tid);
         pre_cell = blockIdx.x;
     }
     cp_async_commit();
@@ -840,18 +863,19 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
         float *d_feat = d_feat_all ? d_feat_all + (size_t)NF * P : nullptr;
         const float *weight = weight_all ? weight_all + P : nullptr;
         const int corner[4] = {cell_corner(cg, 0), cell_corner(cg, 1), cell_corner(cg, 2), cell_corner(cg, 3)};
-        __syncthreads();  // the previous cell's shared data is no longer read
-        for (int i = tid; i < 4 * kLiftHidden; i += kT) (&S.Dpart[0][0])[i] = 0.f;
-        float al[4] = {0.f, 0.f, 0.f, 0.f};  // sum a w_k over the cell (threads < kP)
+        float al[4] = {0.f, 0.f, 0.f, 0.f};  // sum a w_k over the cell (lanes < 16 of the warps 4 i)
         for (int q0 = 0; q0 < npx; q0 += kP) {
-            __syncthreads();
+            // the last chunk of a cell goes in steps of 16 pixels: groups past its
+            // end take no part (their operand columns are not read)
+            const int nk = (min(kP, npx - q0) + 15) >> 4;
+            const bool act = ph < 16 * nk;
             // chunk pixels and their bilinear weights
             if (tid < kP) {
                 const int q = q0 + tid;
                 int pidx = -1;
                 float w[4] = {0.f, 0.f, 0.f, 0.f};
                 if (q < npx) {
-                    const int y = ys + q / nx, x = xs + q % nx;
+                    const int yq = cell_row(cg, q), y = ys + yq, x = xs + q - yq * nx;
                     pidx = y * W + x;
                     const float ax = fminf(fmaxf((float)(2 * x + 1 - (2 * x0 + 1) * patch) * inv2p, 0.f), 1.f);
                     const float ay = fminf(fmaxf((float)(2 * y + 1 - (2 * y0 + 1) * patch) * inv2p, 0.f), 1.f);
@@ -860,62 +884,57 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
                     w[2] = (1.f - ax) * ay;
                     w[3] = ax * ay;
                 }
-                S.pix[tid] = pidx;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) S.w4[tid][k] = w[k];
+                S.pix[buf][tid] = pidx;
+                *reinterpret_cast<float4 *>(&S.w4[tid][0]) = make_float4(w[0], w[1], w[2], w[3]);
             }
-            // this chunk's global inputs were issued a chunk ahead (else now);
-            // the next chunk's go to the other buffer, whose last reader (the
-            // previous chunk) every thread has passed
-            if (pre_cell != cell || pre_q0 != q0) {
+            // this chunk's global inputs were issued a chunk ahead (else now)
+            if (worker && (pre_cell != cell || pre_q0 != q0)) {
                 cp_async_wait<0>();
-                lift_chunk_issue(S, buf, vt, patch, cell, q0, feat_all, d_feat_all, weight_all, E, s, gram, tid);
+                lift_chunk_issue(S, buf, cg, cell, q0, feat_all, d_feat_all, weight_all, E, s, gram, tid);
                 cp_async_commit();
             }
             cp_async_wait<0>();
-            // the previous chunk's Gram MMAs still read the H and b H tiles
+            // F~ as the TF32 hi / lo B tile of Z (pixel rows, channels along K): the
+            // values that this thread copied
+            if (tid < 4 * kP) {
+                const int p = tid & (kP - 1), c0 = 4 * (tid / kP);
+                const float4 v = make_float4(S.Fc[buf][c0][p], S.Fc[buf][c0 + 1][p], S.Fc[buf][c0 + 2][p],
+                                             S.Fc[buf][c0 + 3][p]);
+                put4_tf32(S.FcN[0], S.FcN[1], umma::kmajor_offset(p, c0, 4 * NF, 4), v);
+            }
+            // the previous chunk's Gram and dW1 MMAs still read the H, b H, dZ and F~ tiles
+            bool bad = false;
             if (g_pending) {
-                const bool w_ok = umma::mbar_wait(&S.g_bar, g_phase, kWait);
+                bad = !umma::mbar_wait(&S.g_bar, g_phase, kWait);
                 g_phase ^= 1u;
                 g_pending = false;
-                if (!w_ok) S.abort_flag = 1;
             }
-            __syncthreads();
-            if (S.abort_flag) {
+            umma::fence_async_smem();
+            umma::fence_before();
+            if (__syncthreads_or(bad)) {
+                if (tid == 0) S.abort_flag = 1;
                 ok = false;
                 break;
             }
             umma::fence_after();
-            // F~ as the TF32 hi / lo B tile of Z (pixel rows, channels along K)
-            if (tid >= 128) {
-                const int p = (tid - 128) & (kP - 1);
-#pragma unroll
-                for (int q = (tid - 128) >> 6; q < NF / 4; q += 2) {
-                    const float4 v = make_float4(S.Fc[buf][4 * q][p], S.Fc[buf][4 * q + 1][p], S.Fc[buf][4 * q + 2][p],
-                                                 S.Fc[buf][4 * q + 3][p]);
-                    put4_tf32(S.FcN[0], S.FcN[1], umma::kmajor_offset(p, 4 * q, 4 * NF, 4), v);
-                }
-            }
-            umma::fence_async_smem();
-            __syncthreads();
             // Z = W1 F~ on the tensor cores in 3xTF32 (hi hi + hi lo + lo hi, two K
             // steps of 8, FP32 accumulation in the M H columns, free until M H): its
             // sign decides ReLU', so the operands keep about 22 bits (a BF16 hi / lo
             // split, about 16, flipped enough near-zero units to fail the dF~ bar)
-            if (tid == 0) {
-                umma::fence_after();
-                const uint32_t whi = umma::smem_addr(S.W1A[0]), wlo = umma::smem_addr(S.W1A[1]);
-                const uint32_t fhi = umma::smem_addr(S.FcN[0]), flo = umma::smem_addr(S.FcN[1]);
+            if (!worker) {
+                const uint64_t whi = umma::desc(umma::smem_addr(S.W1A[0]), 4 * NF),
+                               wlo = umma::desc(umma::smem_addr(S.W1A[1]), 4 * NF),
+                               fhi = umma::desc(umma::smem_addr(S.FcN[0]), 4 * NF),
+                               flo = umma::desc(umma::smem_addr(S.FcN[1]), 4 * NF);
+                const uint32_t id = id_z + ((uint32_t)(2 * nk) << 17);
+#pragma unroll
                 for (int ks = 0; ks < NF / 8; ++ks) {
-                    const uint32_t o = 256u * ks;
-                    umma::mma<umma::kTF32>(tmem + cMH, umma::desc(whi + o, 4 * NF), umma::desc(fhi + o, 4 * NF), id_z,
-                                           ks > 0 ? 1u : 0u);
-                    umma::mma<umma::kTF32>(tmem + cMH, umma::desc(whi + o, 4 * NF), umma::desc(flo + o, 4 * NF), id_z,
-                                           1u);
-                    umma::mma<umma::kTF32>(tmem + cMH, umma::desc(wlo + o, 4 * NF), umma::desc(fhi + o, 4 * NF), id_z,
-                                           1u);
+                    const uint64_t o = (256u * ks) >> 4;  // start address field: 16-byte units
+                    umma::mma_warp<umma::kTF32>(tmem + cMH, whi + o, fhi + o, id, ks > 0 ? 1u : 0u);
+                    umma::mma_warp<umma::kTF32>(tmem + cMH, whi + o, flo + o, id, 1u);
+                    umma::mma_warp<umma::kTF32>(tmem + cMH, wlo + o, fhi + o, id, 1u);
                 }
-                umma::commit(&S.mh_bar);
+                umma::commit_warp(&S.mh_bar);
             }
             mh_pending = true;
             // while the Z MMAs run: the next chunk's global inputs to the other
@@ -928,9 +947,11 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
                     nq0 = 0;
                 }
                 pre_cell = -1;
-                if (ncell < n_cells) {
-                    lift_chunk_issue(S, buf ^ 1, vt, patch, ncell, nq0, feat_all, d_feat_all, weight_all, E, s, gram,
-                                     tid);
+                if (worker && ncell < n_cells) {
+                    CellGeo ng = cg;
+                    if (ncell != cell) ng = cell_geo(S, vt, patch, ncell);
+                    lift_chunk_issue(S, buf ^ 1, ng, ncell, nq0, feat_all, d_feat_all, weight_all,
+                                     E, s, gram, tid);
                     pre_cell = ncell;
                     pre_q0 = nq0;
                 }
@@ -938,126 +959,115 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
             }
             // F~ as the BF16 hi / lo B tile of dW1 (channel rows, pixels along K);
             // the previous chunk's dW1 MMAs, which read it, completed with the Gram's
-            if (d_w1 && tid < 128) {
-                const int c = tid >> 3, p8 = 8 * (tid & 7);
+            if (d_w1 && tid >= kT - 128 && worker) {
+                const int t = tid - (kT - 128), c = t >> 3, p8 = 8 * (t & 7);
                 const float4 f0 = *reinterpret_cast<const float4 *>(&S.Fc[buf][c][p8]);
                 const float4 f1 = *reinterpret_cast<const float4 *>(&S.Fc[buf][c][p8 + 4]);
                 const float v[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
                 put8_split(reinterpret_cast<unsigned char *>(S.FcT[0]), reinterpret_cast<unsigned char *>(S.FcT[1]),
                            umma::kmajor_offset(c, p8, 2 * kP, 2), v);
             }
-            {
-                const bool w_ok = umma::mbar_wait(&S.mh_bar, mh_phase, kWait);
-                if (w_ok) {
-                    mh_phase ^= 1u;
-                    mh_pending = false;
-                }
-                if (__syncthreads_or(!w_ok)) {
-                    if (tid == 0) S.abort_flag = 1;
-                    ok = false;
-                    break;
-                }
+            // a wait that gives up is voted on at the next barrier
+            bad = !umma::mbar_wait(&S.mh_bar, mh_phase, kWait);
+            if (!bad) {
+                mh_phase ^= 1u;
+                mh_pending = false;
             }
             umma::fence_after();
-            // H = relu(Z + b1) of (jt, pixel half): registers, the Gram A tile
+            // H = relu(Z + b1) of (jt, pixel group): registers, the Gram A tile
             // (row jt) and M H's B tile
-            float hv[32];
-            {
+            float hv[16];
+            if (act) {
                 const float bj = S.b1[jt];
-                float t16[16];
-                umma::tmem_ld16(lane_addr + cMH + ph, t16);
+                umma::tmem_ld16(lane_addr + cMH + ph, hv);
 #pragma unroll
-                for (int t = 0; t < 16; ++t) hv[t] = fmaxf(t16[t] + bj, 0.f);
-                umma::tmem_ld16(lane_addr + cMH + ph + 16, t16);
+                for (int t = 0; t < 16; ++t) hv[t] = fmaxf(hv[t] + bj, 0.f);
+                uint32_t hi[8], lo[8];
 #pragma unroll
-                for (int t = 0; t < 16; ++t) hv[16 + t] = fmaxf(t16[t] + bj, 0.f);
-            }
-            {
-                uint32_t hi[16], lo[16];
+                for (int t = 0; t < 8; ++t) split2_bf16(hv[2 * t], hv[2 * t + 1], hi[t], lo[t]);
+                umma::tmem_st8(lane_addr + cHAhi + ph / 2, hi);
+                umma::tmem_st8(lane_addr + cHAlo + ph / 2, lo);
+                // H as M H's B tile, pixel rows of 8 straight from the registers
 #pragma unroll
-                for (int t = 0; t < 16; ++t) split2_bf16(hv[2 * t], hv[2 * t + 1], hi[t], lo[t]);
-                umma::tmem_st16(lane_addr + cHAhi + ph / 2, hi);
-                umma::tmem_st16(lane_addr + cHAlo + ph / 2, lo);
+                for (int q = 0; q < 2; ++q) {
+                    const uint32_t o = hb_mn_offset(jt, ph + 8 * q);
+                    *reinterpret_cast<uint4 *>(op + oHBhi + o) =
+                        make_uint4(hi[4 * q], hi[4 * q + 1], hi[4 * q + 2], hi[4 * q + 3]);
+                    *reinterpret_cast<uint4 *>(op + oHBlo + o) =
+                        make_uint4(lo[4 * q], lo[4 * q + 1], lo[4 * q + 2], lo[4 * q + 3]);
+                }
                 umma::tmem_st_wait();
-            }
-            // H as M H's B tile, pixel rows of 8 straight from the registers
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float v[8] = {hv[8 * q],     hv[8 * q + 1], hv[8 * q + 2], hv[8 * q + 3],
-                                    hv[8 * q + 4], hv[8 * q + 5], hv[8 * q + 6], hv[8 * q + 7]};
-                put8_split(op + oHBhi, op + oHBlo, hb_mn_offset(jt, ph + 8 * q), v);
             }
             umma::fence_before();
             umma::fence_async_smem();
-            __syncthreads();
+            if (__syncthreads_or(bad)) {
+                if (tid == 0) S.abort_flag = 1;
+                ok = false;
+                break;
+            }
             // M H on the tensor cores
-            if (tid == 0) {
+            if (!worker) {
                 umma::fence_after();
-                for (int pass = 0; pass < 3; ++pass) {
-                    const uint32_t a = tmem + (pass == 2 ? cMlo : cMhi), b = sop + (pass == 1 ? oHBlo : oHBhi);
+                const uint32_t id = (id_mh + ((uint32_t)(2 * nk) << 17)) | (1u << 16);
+                const uint64_t bhi = desc_strides(sop + oHBhi, 1024, 128), blo = desc_strides(sop + oHBlo, 1024, 128);
+#pragma unroll
+                for (int pass = 0; pass < 3; ++pass)
+#pragma unroll
                     for (int ks = 0; ks < kLiftHidden / 16; ++ks)
-                        umma::mma_f16_ts(tmem + cMH, a + 8u * ks, desc_strides(b + 2048u * ks, 1024, 128),
-                                         id_mh | (1u << 16), (pass > 0 || ks > 0) ? 1u : 0u);
-                }
-                umma::commit(&S.mh_bar);
+                        umma::mma_f16_ts_warp(tmem + cMH, tmem + (pass == 2 ? cMlo : cMhi) + 8u * ks,
+                                              (pass == 1 ? blo : bhi) + 128u * ks, id, (pass > 0 || ks > 0) ? 1u : 0u);
+                umma::commit_warp(&S.mh_bar);
             }
             mh_pending = true;
             const float e0 = S.E[buf][0][jt], e1 = S.E[buf][1][jt], e2 = S.E[buf][2][jt], e3 = S.E[buf][3][jt],
                         uj = S.u[jt];
-            auto e_at = [&](int t) {
-                const float4 w = *reinterpret_cast<const float4 *>(&S.w4[ph + t][0]);
-                return w.x * e0 + w.y * e1 + w.z * e2 + w.w * e3;
-            };
             // per pixel over this warp's 32 hidden units: H.e (while the M H
             // MMAs run), then H.(M H + 2 u), the two sums the cosine needs
             // (|F^|^2 = H.M H + 2 u.H + |b2|^2)
-            {
-                float v[32];
+            if (act) {
+                float v[16];
 #pragma unroll
-                for (int t = 0; t < 32; ++t) v[t] = hv[t] * e_at(t);
-                red[((warp & 3) * kP + ph + lane) * 2 + 0] = warp_rs32(v, lane);
+                for (int t = 0; t < 16; ++t) {
+                    const float4 w = *reinterpret_cast<const float4 *>(&S.w4[ph + t][0]);
+                    v[t] = hv[t] * (w.x * e0 + w.y * e1 + w.z * e2 + w.w * e3);
+                }
+                const float r = warp_rs16(v, lane);
+                if (lane < 16) red[((warp & 3) * kP + ph + lane) * 2 + 0] = r;
             }
-            {
-                const bool w_ok = umma::mbar_wait(&S.mh_bar, mh_phase, kWait);
-                if (w_ok) {
-                    mh_phase ^= 1u;
-                    mh_pending = false;
-                }
-                if (__syncthreads_or(!w_ok)) {
-                    if (tid == 0) S.abort_flag = 1;
-                    ok = false;
-                    break;
-                }
+            bad = !umma::mbar_wait(&S.mh_bar, mh_phase, kWait);
+            if (!bad) {
+                mh_phase ^= 1u;
+                mh_pending = false;
             }
             umma::fence_after();
-            // thread (jt, pixel half ph): its M H row, the corner terms
-            float mh[32];
-            {
-                float t16[16];
-                umma::tmem_ld16(lane_addr + cMH + ph, t16);
+            // thread (jt, pixel group ph): its M H row, the corner terms
+            float mh[16];
+            if (act) {
+                umma::tmem_ld16(lane_addr + cMH + ph, mh);
+                float v[16];
 #pragma unroll
-                for (int t = 0; t < 16; ++t) mh[t] = t16[t];
-                umma::tmem_ld16(lane_addr + cMH + ph + 16, t16);
-#pragma unroll
-                for (int t = 0; t < 16; ++t) mh[16 + t] = t16[t];
+                for (int t = 0; t < 16; ++t) v[t] = hv[t] * fmaf(2.f, uj, mh[t]);
+                const float r = warp_rs16(v, lane);
+                if (lane < 16) red[((warp & 3) * kP + ph + lane) * 2 + 1] = r;
             }
-            {
-                float v[32];
-#pragma unroll
-                for (int t = 0; t < 32; ++t) v[t] = hv[t] * fmaf(2.f, uj, mh[t]);
-                red[((warp & 3) * kP + ph + lane) * 2 + 1] = warp_rs32(v, lane);
+            if (__syncthreads_or(bad)) {
+                if (tid == 0) S.abort_flag = 1;
+                ok = false;
+                break;
             }
-            __syncthreads();
-            // per pixel: cosine, loss, a_p, b_p
-            if (tid < kP) {
-                const int p = tid;
+            // per pixel: cosine, loss, a_p, b_p; the four warps of a pixel group
+            // each for themselves (no barrier), one of them into the sums
+            if (act && lane < 16) {
+                const int p = ph + lane;
                 float de = 0.f, dmu = 0.f;
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
-                    de += red[(b * kP + p) * 2 + 0];
-                    dmu += red[(b * kP + p) * 2 + 1];
+                    const float2 r = *reinterpret_cast<const float2 *>(&red[(b * kP + p) * 2]);
+                    de += r.x;
+                    dmu += r.y;
                 }
-                const float *w = S.w4[p];
+                const float4 w4 = *reinterpret_cast<const float4 *>(&S.w4[p][0]);
+                const float w[4] = {w4.x, w4.y, w4.z, w4.w};
                 const float *sS = S.sS[buf], *sG = S.sG[buf];
                 const float dot = de + w[0] * sS[0] + w[1] * sS[1] + w[2] * sS[2] + w[3] * sS[3];
                 const float nF2 = w[0] * w[0] * sG[0] + w[1] * w[1] * sG[4] + w[2] * w[2] * sG[7] +
@@ -1066,37 +1076,35 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
                                          w[1] * w[2] * sG[5] + w[1] * w[3] * sG[6] + w[2] * w[3] * sG[8]);
                 const float nFh2 = dmu + bt;
                 float a = 0.f, b = 0.f;
-                const int pidx = S.pix[p];
-                if (pidx >= 0) {
+                if (S.pix[buf][p] >= 0) {
                     const bool okp = nF2 > 0.f && nFh2 > 0.f;
                     const float wpx = weight ? S.wpx[buf][p] : 1.f;
                     const float g = g0 * wpx;
                     const float inv = okp ? rsqrtf(nF2) * rsqrtf(nFh2) : 0.f;
                     const float cs = dot * inv;
-                    t_loss += wpx * (1.f - cs);
                     a = -g * inv;
                     b = okp ? g * cs / nFh2 : 0.f;
-                    t_sb += b;
+                    if ((warp & 3) == 0) {
+                        t_loss += wpx * (1.f - cs);
+                        t_sb += b;
+                    }
                 }
-                S.ab[p][0] = a;
-                S.ab[p][1] = b;
+                *reinterpret_cast<float4 *>(&S.ab[warp][lane][0]) = make_float4(a * w[0], a * w[1], a * w[2], a * w[3]);
+                S.ab[warp][lane][4] = b;
+                if ((warp & 3) == 0)
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    S.aw[p][k] = a * w[k];
-                    al[k] += a * w[k];
-                }
+                    for (int k = 0; k < 4; ++k) al[k] += a * w[k];
             }
-            __syncthreads();
+            __syncwarp();
             // dZ (to Hh), b H (to the Gram B tile), db1, hb and D of the corners
-            // (thread jt over its pixel half)
-            {
+            // (thread jt over its pixel group)
+            if (act) {
                 float Dk[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-                for (int t = 0; t < 32; ++t) {
-                    const int p = ph + t;
+                for (int t = 0; t < 16; ++t) {
                     // dL/dH = a e_p + b (M H + u), a e_p = sum_k (a w_k) e_k
-                    const float bp = S.ab[p][1];
-                    const float4 awp = *reinterpret_cast<const float4 *>(&S.aw[p][0]);
+                    const float bp = S.ab[warp][t][4];
+                    const float4 awp = *reinterpret_cast<const float4 *>(&S.ab[warp][t][0]);
                     const float dh =
                         fmaf(awp.x, e0, fmaf(awp.y, e1, fmaf(awp.z, e2, fmaf(awp.w, e3, bp * (mh[t] + uj)))));
                     const float dz = hv[t] > 0.f ? dh : 0.f;
@@ -1110,23 +1118,23 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
                     hv[t] *= bp;
                 }
 #pragma unroll
-                for (int t4 = 0; t4 < 8; ++t4)
+                for (int t4 = 0; t4 < 4; ++t4)
                     *reinterpret_cast<float4 *>(&S.Hh[jt][ph + 4 * t4]) =
                         make_float4(mh[4 * t4], mh[4 * t4 + 1], mh[4 * t4 + 2], mh[4 * t4 + 3]);
 #pragma unroll
-                for (int c8 = 0; c8 < 4; ++c8) {
+                for (int c8 = 0; c8 < 2; ++c8) {
                     const float v[8] = {hv[8 * c8],     hv[8 * c8 + 1], hv[8 * c8 + 2], hv[8 * c8 + 3],
                                         hv[8 * c8 + 4], hv[8 * c8 + 5], hv[8 * c8 + 6], hv[8 * c8 + 7]};
                     put8_split(op + oBHhi, op + oBHlo, umma::kmajor_offset(jt, ph + 8 * c8, 2 * kP, 2), v);
                 }
 #pragma unroll
-                for (int k = 0; k < 4; ++k) atomicAdd(&S.Dpart[k][jt], Dk[k]);
+                for (int k = 0; k < 4; ++k) S.Dpart[warp >> 2][k][jt] += Dk[k];
                 if (d_w1) {  // dZ as the A operand of dW1 (row jt, pixel pairs)
-                    uint32_t hi[16], lo[16];
+                    uint32_t hi[8], lo[8];
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) split2_bf16(mh[2 * q], mh[2 * q + 1], hi[q], lo[q]);
-                    umma::tmem_st16(lane_addr + cDZhi + ph / 2, hi);
-                    umma::tmem_st16(lane_addr + cDZlo + ph / 2, lo);
+                    for (int q = 0; q < 8; ++q) split2_bf16(mh[2 * q], mh[2 * q + 1], hi[q], lo[q]);
+                    umma::tmem_st8(lane_addr + cDZhi + ph / 2, hi);
+                    umma::tmem_st8(lane_addr + cDZlo + ph / 2, lo);
                     umma::tmem_st_wait();
                 }
             }
@@ -1134,98 +1142,110 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
             umma::fence_async_smem();
             __syncthreads();
             // Gram += H (b H)^T on the tensor cores, left running
-            if (tid == kGramTid) {
+            if (!worker) {
                 umma::fence_after();
-                for (int pass = 0; pass < 3; ++pass) {
-                    const uint32_t a = tmem + (pass == 2 ? cHAlo : cHAhi), b = sop + (pass == 1 ? oBHlo : oBHhi);
-                    for (int ks = 0; ks < kP / 16; ++ks)
-                        umma::mma_f16_ts(tmem + cG, a + 8u * ks, umma::desc(b + 256u * ks, 2 * kP), id_g,
-                                         (g_started || pass > 0 || ks > 0) ? 1u : 0u);
+                const uint64_t bhi = umma::desc(sop + oBHhi, 2 * kP), blo = umma::desc(sop + oBHlo, 2 * kP);
+                const uint64_t fhi = umma::desc(umma::smem_addr(S.FcT[0]), 2 * kP),
+                               flo = umma::desc(umma::smem_addr(S.FcT[1]), 2 * kP);
+                const uint32_t acc0 = g_started ? 1u : 0u;
+#pragma unroll
+                for (int ks = 0; ks < kP / 16; ++ks) {
+                    if (ks >= nk) break;
+#pragma unroll
+                    for (int pass = 0; pass < 3; ++pass)
+                        umma::mma_f16_ts_warp(tmem + cG, tmem + (pass == 2 ? cHAlo : cHAhi) + 8u * ks,
+                                              (pass == 1 ? blo : bhi) + 16u * ks, id_g,
+                                              (pass > 0 || ks > 0) ? 1u : acc0);
+                    // dW1 += dZ F~^T: A = dZ in TMEM, B = the F~ tile, accumulated over the CTA's chunks
+                    if (d_w1)
+#pragma unroll
+                        for (int pass = 0; pass < 3; ++pass)
+                            umma::mma_f16_ts_warp(tmem + cDW, tmem + (pass == 2 ? cDZlo : cDZhi) + 8u * ks,
+                                                  (pass == 1 ? flo : fhi) + 16u * ks, id_dw,
+                                                  (pass > 0 || ks > 0) ? 1u : acc0);
                 }
-                // dW1 += dZ F~^T: A = dZ in TMEM, B = the F~ tile, accumulated over the CTA's chunks
-                if (d_w1) {
-                    const uint32_t fhi = umma::smem_addr(S.FcT[0]), flo = umma::smem_addr(S.FcT[1]);
-                    for (int pass = 0; pass < 3; ++pass) {
-                        const uint32_t a = tmem + (pass == 2 ? cDZlo : cDZhi), b = pass == 1 ? flo : fhi;
-                        for (int ks = 0; ks < kP / 16; ++ks)
-                            umma::mma_f16_ts(tmem + cDW, a + 8u * ks, umma::desc(b + 256u * ks, 2 * kP), id_dw,
-                                             (g_started || pass > 0 || ks > 0) ? 1u : 0u);
-                    }
-                }
-                umma::commit(&S.g_bar);
+                umma::commit_warp(&S.g_bar);
             }
             g_started = true;
             g_pending = true;
             if (d_feat) {
-                // dF~ = W1^T dZ: each warp sums a range of hidden units for all
-                // channels of lane l's pixels 2 l and 2 l + 1, channel pairs packed
-                // (the warp that issued the Gram and dW1 MMAs takes 2 units, the
-                // other seven 18); W1 rows come in warp-uniform loads, and the eight
-                // warps' partial sums meet in the M H operand tile, free until the
-                // next chunk
-                constexpr int kIssueWarp = kGramTid / 32, kShort = 2, kLong = (kLiftHidden - kShort) / 7;
-                static_assert(7 * kLong + kShort == kLiftHidden, "hidden units over the dF~ warps");
-                const int j0 = warp < kIssueWarp ? kLong * warp : warp == kIssueWarp ? kLong * warp
-                                                                                     : kLong * (warp - 1) + kShort;
-                const int nj = warp == kIssueWarp ? kShort : kLong;
-                f2 acc[NF / 2][2];  // [channel pair][pixel]
+                // dF~ = W1^T dZ: warps w and w + 8 sum 16 hidden units, 32 pixels each;
+                // lane l four pixels and four channels in packed channel pairs (a
+                // 16-byte load of dZ and one of W1, each shared by a quarter of the
+                // lanes or more, feed eight FMAs); the partial sums meet in the M H
+                // operand tile, free until the next chunk
+                constexpr int kUnits = kLiftHidden / 8;
+                const int wg = warp & 7, c0 = 4 * (lane >> 3), p4 = 32 * (warp >> 3) + 4 * (lane & 7);
+                float *part = reinterpret_cast<float *>(op + oHBhi);  // [8 unit ranges][NF][kP]
+                // (a short last chunk: only the pixels that it holds)
+                if (worker && p4 < 16 * nk) {
+                    f2 acc[2][4];  // [channel pair][pixel]
 #pragma unroll
-                for (int k = 0; k < NF / 2; ++k) acc[k][0] = acc[k][1] = 0ull;
-#pragma unroll 2
-                for (int jj = 0; jj < nj; ++jj) {
-                    const int j = j0 + jj;
-                    const float2 dz = *reinterpret_cast<const float2 *>(&S.Hh[j][2 * lane]);
-                    const f2 d0 = f2_make(dz.x, dz.x), d1 = f2_make(dz.y, dz.y);
+                    for (int y = 0; y < 4; ++y) acc[0][y] = acc[1][y] = 0ull;
+#pragma unroll 4
+                    for (int jj = 0; jj < kUnits; ++jj) {
+                        const int j = kUnits * wg + jj;
+                        const float4 dz = *reinterpret_cast<const float4 *>(&S.Hh[j][p4]);
+                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&S.W1r[j][c0]);
+                        const f2 d[4] = {f2_make(dz.x, dz.x), f2_make(dz.y, dz.y), f2_make(dz.z, dz.z),
+                                         f2_make(dz.w, dz.w)};
 #pragma unroll
-                    for (int k4 = 0; k4 < NF / 4; ++k4) {
-                        const ulonglong2 w = *reinterpret_cast<const ulonglong2 *>(&S.W1r[j][4 * k4]);
-                        acc[2 * k4][0] = f2_fma(w.x, d0, acc[2 * k4][0]);
-                        acc[2 * k4][1] = f2_fma(w.x, d1, acc[2 * k4][1]);
-                        acc[2 * k4 + 1][0] = f2_fma(w.y, d0, acc[2 * k4 + 1][0]);
-                        acc[2 * k4 + 1][1] = f2_fma(w.y, d1, acc[2 * k4 + 1][1]);
+                        for (int y = 0; y < 4; ++y) {
+                            acc[0][y] = f2_fma(w.x, d[y], acc[0][y]);
+                            acc[1][y] = f2_fma(w.y, d[y], acc[1][y]);
+                        }
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        float e[4], o[4];  // channels c0 + 2 k and + 1
+#pragma unroll
+                        for (int y = 0; y < 4; ++y) f2_split(acc[k][y], e[y], o[y]);
+                        float *pk = &part[(wg * NF + c0 + 2 * k) * kP + p4];
+                        *reinterpret_cast<float4 *>(pk) = make_float4(e[0], e[1], e[2], e[3]);
+                        *reinterpret_cast<float4 *>(pk + kP) = make_float4(o[0], o[1], o[2], o[3]);
                     }
                 }
-                float *part = reinterpret_cast<float *>(op + oHBhi);  // [8 warps][NF][kP]
-#pragma unroll
-                for (int k = 0; k < NF / 2; ++k) {
-                    float a0, b0, a1, b1;  // (channel 2 k, 2 k + 1) at pixels 2 l and 2 l + 1
-                    f2_split(acc[k][0], a0, b0);
-                    f2_split(acc[k][1], a1, b1);
-                    *reinterpret_cast<float2 *>(&part[(warp * NF + 2 * k) * kP + 2 * lane]) = make_float2(a0, a1);
-                    *reinterpret_cast<float2 *>(&part[(warp * NF + 2 * k + 1) * kP + 2 * lane]) = make_float2(b0, b1);
-                }
                 __syncthreads();
-                // thread t: channel t / 16, pixels 4 (t % 16) + [0, 4)
-                const int c = tid >> 4, p0 = 4 * (tid & 15);
-                const float4 d4 = *reinterpret_cast<const float4 *>(&S.dF0[buf][c][p0]);
-                float sum[4] = {0.f, 0.f, 0.f, 0.f};
+                // thread t: channel t / 32, pixels 2 (t % 32) + [0, 2)
+                const int c = tid >> 5, p0 = 2 * lane;
+                const int2 px = *reinterpret_cast<const int2 *>(&S.pix[buf][p0]);
+                if (worker && px.x >= 0) {  // a chunk's pixels come first
+                    const float2 d2 = *reinterpret_cast<const float2 *>(&S.dF0[buf][c][p0]);
+                    float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
-                for (int w = 0; w < 8; ++w) {
-                    const float4 v = *reinterpret_cast<const float4 *>(&part[(w * NF + c) * kP + p0]);
-                    sum[0] += v.x;
-                    sum[1] += v.y;
-                    sum[2] += v.z;
-                    sum[3] += v.w;
-                }
-                const float o[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-                for (int y = 0; y < 4; ++y) {
-                    const int pidx = S.pix[p0 + y];
-                    if (pidx >= 0) d_feat[(size_t)c * HW + pidx] = o[y] + sum[y];
+                    for (int w = 0; w < 8; ++w) {
+                        const float2 v = *reinterpret_cast<const float2 *>(&part[(w * NF + c) * kP + p0]);
+                        sum.x += v.x;
+                        sum.y += v.y;
+                    }
+                    d_feat[(size_t)c * HW + px.x] = d2.x + sum.x;
+                    if (px.y >= 0) d_feat[(size_t)c * HW + px.y] = d2.y + sum.y;
                 }
             }
             buf ^= 1;
         }
         if (!ok) break;
-        __syncthreads();
-        // the cell's D rows and alpha
-        for (int i = tid; i < 4 * kLiftHidden; i += kT) {
-            const int k = i / kLiftHidden, j = i - k * kLiftHidden;
-            if (npx > 0) atomicAdd(D + (size_t)corner[k] * kLiftHidden + j, S.Dpart[k][j]);
-        }
-        if (tid < kP && npx > 0)
+        // the cell's D rows (thread t: corner t / 128, unit t % 128; summed over the
+        // pixel groups and cleared: added to before the last chunk's barriers, and
+        // again after the next chunk's first) and alpha
+        if (worker && npx > 0) {
+            static_assert(kT == 4 * kLiftHidden, "one value of D a thread");
+            float d = 0.f;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) atomicAdd(alpha + corner[k], al[k]);
+            for (int g = 0; g < 4; ++g) {
+                d += S.Dpart[g][warp >> 2][jt];
+                S.Dpart[g][warp >> 2][jt] = 0.f;
+            }
+            atomicAdd(D + (size_t)cell_corner(cg, warp >> 2) * kLiftHidden + jt, d);
+            if ((warp & 3) == 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+#pragma unroll
+                    for (int o = 8; o > 0; o >>= 1) al[k] += __shfl_xor_sync(0xffffffffu, al[k], o);
+                    if (lane == 0) atomicAdd(alpha + corner[k], al[k]);
+                }
+            }
+        }
     }
     cp_async_wait<0>();  // no copy still writes shared memory
     // the last Gram MMAs (and an M H that a wait gave up on), then the CTA's sums
@@ -1238,10 +1258,10 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
     __syncthreads();
     umma::fence_after();
     ok = ok && !S.abort_flag;
-    if (ok && g_started) {
-        // Gram (symmetric): thread jt, the half of the columns its warp's pixel half names
+    if (ok && worker && g_started) {
+        // Gram (symmetric): thread jt, the quarter of the columns its warp's pixel group names
 #pragma unroll 1
-        for (int c0 = 0; c0 < kLiftHidden / 2; c0 += 16) {
+        for (int c0 = 0; c0 < kLiftHidden / 4; c0 += 16) {
             float d[16];
             umma::tmem_ld16(lane_addr + cG + 2 * ph + c0, d);
 #pragma unroll
@@ -1249,7 +1269,7 @@ __global__ void __launch_bounds__(lt::kT, 1) k_lift_tc(
         }
     }
     if (!ok && tid == 0 && err) atomicExch(err, 1);
-    if (ok) {
+    if (ok && worker) {
         atomicAdd(hb_out + jt, hb);
         if (d_b1) atomicAdd(d_b1 + jt, db1);
         if (d_w1 && g_started && warp < 4) {  // dW1 row jt from TMEM
@@ -1352,7 +1372,7 @@ cudaError_t lift_all(int num_sms, cudaStream_t st, const ViewTable &vt, int nf, 
         // one CTA per SM: it holds all 512 TMEM columns
         if (smem > 227 * 1024 || 2 * (smem + 1024) <= 228 * 1024) return cudaErrorInvalidConfiguration;
         cudaFuncSetAttribute(k_lift_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        k_lift_tc<<<grid_ctas, lt::kT, smem, st>>>(vt, np, patch, feat, w1, b1, M, E, sv, u, beta, gram, weight, g,
+        k_lift_tc<<<grid_ctas, lt::kAll, smem, st>>>(vt, np, patch, feat, w1, b1, M, E, sv, u, beta, gram, weight, g,
                                                    loss, D, alpha, sb, hb, Gb, d_w1, d_b1, d_feat, err);
     } else if (nf == 32) {
         // the BF16 operand tiles and the FP32 arrays of N_l = 32 exceed shared memory: all FP32 on the CUDA cores
