@@ -2,8 +2,7 @@
 // and transmittance (Eq. 3, Eq. 10), the per-pixel weighted loss (Eq. 4 /
 // Eq. 14), and the reverse-order blending backward.
 //
-// One CTA per 16x16 image tile, PX pixels per thread (forward 2; backward 4
-// for up to 16 feature channels, 2 for 32: registers).  The tile's
+// One CTA per 16x16 image tile, PX pixels per thread (forward 2; backward 4).  The tile's
 // depth-ordered Gaussian list is staged in shared memory in batches of list
 // entries by the bulk-copy (TMA) engine: one cp.async.bulk per attribute
 // record of an entry, completed on the batch's mbarrier, in a ring of stages
@@ -114,13 +113,13 @@ __device__ __forceinline__ TileP<PX> tilep(const ViewTable &vt) {
     return c;
 }
 
-// pixels per thread: forward 2; backward 4 up to 16 feature channels (the
-// per-Gaussian warp reduction is shared by more pixels), 2 for 32 (registers)
+// pixels per thread: forward 2; backward 4 (the per-Gaussian warp reduction is
+// shared by more pixels)
 #ifndef UPS_FWD_PX
 #define UPS_FWD_PX 2
 #endif
 __host__ __device__ constexpr int blend_px_fwd(int nf) { return UPS_FWD_PX; }
-__host__ __device__ constexpr int blend_px_bwd(int nf) { return nf <= 16 ? 4 : 2; }
+__host__ __device__ constexpr int blend_px_bwd(int nf) { return 4; }
 
 // Exponent coefficients of a staged Gaussian for a thread's pixel column, in
 // base 2: exp(p) = 2^(p log2 e), so the coefficients carry the factor log2 e
@@ -389,20 +388,16 @@ __global__ void k_scale_mean(const float4 *__restrict__ scale, size_t n, float c
 // backward
 // ---------------------------------------------------------------------------
 
-#ifndef UPS_BWD_STAGES
-#define UPS_BWD_STAGES 3
-#endif
-constexpr int kBwdStages = UPS_BWD_STAGES;
-// Tuning of the backward (compile-time): CTAs per SM the register allocation
-// targets at 4 pixels per thread (8 caps registers at 128), and whether a warp
-// skips a pixel row no lane of it blends (a vote per row) or runs it masked.
-#ifndef UPS_BWD_MIN_BLOCKS
-#define UPS_BWD_MIN_BLOCKS 6
-#endif
-#ifndef UPS_BWD_ROW_SKIP
-#define UPS_BWD_ROW_SKIP 0
-#endif
-constexpr int kBwdMinBlocks = UPS_BWD_MIN_BLOCKS;
+// Ring depth and the CTAs per SM that the registers are cut for.  Up to 16 feature
+// channels 8 CTAs of two warps (128 registers, 52 bytes spilled, a ring of 2): on
+// batches of many waves as fast as 6 (156 registers, a ring of 3; 1.84 ms for
+// 8 x 640x480 at 16 channels either way), but a frame of 1200 tiles fits the GPU at
+// once (0.277 against 0.320 ms).  At 32 channels the 128 registers of dL/dF of four
+// pixels leave 4 CTAs of 234 registers: 5.88 ms for 8 x 1280x720, two pixels a
+// thread 7.61 ms (its warps reduce every Gaussian's 44 sums for half the pixels);
+// batches of 32 entries 6.19 ms, 5 CTAs (spills) 7.16 ms.
+constexpr int bwd_stages(int nf) { return nf <= 16 ? 2 : 3; }
+constexpr int bwd_ctas(int nf) { return nf <= 16 ? 8 : 4; }
 constexpr int kRedStride = 36;  // floats per lane row of the reduction scratch
 
 // Sums over the warp of the per-lane gradient record values v (float4 groups
@@ -446,7 +441,7 @@ __device__ __forceinline__ void warp_record_add(const float4 (&v)[NG], float (*r
 }
 
 template <int NF, int PX>
-__global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_composite_bwd(
+__global__ void __launch_bounds__(Px<PX>::NT, bwd_ctas(NF)) k_composite_bwd(
     ViewTable vt, BlendParams bp, int N, int per_view, const uint2 *__restrict__ ranges,
     const uint32_t *__restrict__ ival, const float4 *__restrict__ xyzo,
     const float4 *__restrict__ conic, const float4 *__restrict__ color,
@@ -454,8 +449,8 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
     const uint32_t *__restrict__ in_nc, const float *__restrict__ dC,
     const float *__restrict__ dD, const float *__restrict__ dF, const float *__restrict__ dT,
     float *__restrict__ g2, uint32_t *__restrict__ hits, int *__restrict__ err) {
-    constexpr int NT = Px<PX>::NT, RS = Px<PX>::RS, NW = NT / 32, NS = kBwdStages;
-    constexpr int KB = NF > 16 ? 32 : UPS_BWD_BATCH;
+    constexpr int NT = Px<PX>::NT, RS = Px<PX>::RS, NW = NT / 32, NS = bwd_stages(NF);
+    constexpr int KB = UPS_BWD_BATCH;
     constexpr int STRIDE = kG2Base + NF;  // record floats, a multiple of 4
     constexpr int NG = STRIDE / 4;
     static_assert(NT >= KB, "one thread per staged entry");
@@ -531,9 +526,7 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
         for (int b0 = 0; b0 < NS; ++b0)
             if (b0 < issued) issue(b0, pg[b0]);
     }
-    float fy[PX];
-#pragma unroll
-    for (int q = 0; q < PX; ++q) fy[q] = (float)(tc.py0 + RS * q);
+    const float fy0 = (float)tc.py0;
     int b = 0;
     for (; b < nb; ++b) {
         const uint32_t nxt = issued < nb ? entry_gv(issued) : 0u;
@@ -557,7 +550,7 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
             bool any = false;
 #pragma unroll
             for (int q = 0; q < PX; ++q) {
-                dy[q] = fy[q] - g.y;
+                dy[q] = (fy0 + (float)(RS * q)) - g.y;  // whole numbers: the forward's difference
                 G[q] = falloff(expo_at(ex, dy[q]));
                 alpha[q] = fminf(bp.alpha_max, g.w * G[q]);
                 use[q] = idx < (int)nc[q] && alpha[q] >= bp.alpha_min;
@@ -566,13 +559,6 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
             if (!__any_sync(0xffffffffu, any)) continue;
             const float4 col = S.color[j];
             const f2 ca = f2_make(col.x, col.y), cb = f2_make(col.z, g.z);
-            f2 fj[NF > 0 ? NF / 2 : 1];
-#pragma unroll
-            for (int c = 0; c < NF; c += 4) {
-                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(&S.feat[j][c]);
-                fj[c / 2] = f.x;
-                fj[c / 2 + 1] = f.y;
-            }
             // per-thread sums over its pixels.  With t = dL/dalpha * G for an
             // unclamped alpha (0 otherwise), dL/do = sum t and the exponent
             // p = pa + dy (pb + pc dy) has dL/dp = o t per pixel, so the conic
@@ -583,33 +569,46 @@ __global__ void __launch_bounds__(Px<PX>::NT, PX == 4 ? kBwdMinBlocks : 1) k_com
             f2 vF[NF > 0 ? NF / 2 : 1];
 #pragma unroll
             for (int c = 0; c < NF / 2; ++c) vF[c] = 0ull;
+            // weights, transmittances and the colour part of every pixel, then the
+            // features four channels at a time for all pixels (a staged feature is
+            // read once and not held), then dL/dalpha
+            float rom[PX], w[PX];
+            f2 w2[PX], xg2[PX];
 #pragma unroll
             for (int q = 0; q < PX; ++q) {
-                if (UPS_BWD_ROW_SKIP && !__any_sync(0xffffffffu, use[q])) continue;
                 const float a = use[q] ? alpha[q] : 0.f;
-                const float rom = use[q] ? __fdividef(1.f, 1.f - a) : 1.f;
-                T[q] *= rom;  // transmittance in front of this Gaussian
-                const float w = a * T[q];
-                const f2 w2 = f2_make(w, w);
-                f2 xg2 = f2_fma(cb, gCb[q], f2_fma(ca, gCa[q], 0ull));
+                rom[q] = use[q] ? __fdividef(1.f, 1.f - a) : 1.f;
+                T[q] *= rom[q];  // transmittance in front of this Gaussian
+                w[q] = a * T[q];
+                w2[q] = f2_make(w[q], w[q]);
+                xg2[q] = f2_fma(cb, gCb[q], f2_fma(ca, gCa[q], 0ull));
+                sca = f2_fma(w2[q], gCa[q], sca);
+                scb = f2_fma(w2[q], gCb[q], scb);
+            }
 #pragma unroll
-                for (int c = 0; c < NF / 2; ++c) {
-                    xg2 = f2_fma(fj[c], gF[q][c], xg2);
-                    vF[c] = f2_fma(w2, gF[q][c], vF[c]);
+            for (int c = 0; c < NF / 2; c += 2) {
+                const ulonglong2 f = *reinterpret_cast<const ulonglong2 *>(&S.feat[j][2 * c]);
+#pragma unroll
+                for (int q = 0; q < PX; ++q) {
+                    xg2[q] = f2_fma(f.x, gF[q][c], xg2[q]);
+                    vF[c] = f2_fma(w2[q], gF[q][c], vF[c]);
+                    xg2[q] = f2_fma(f.y, gF[q][c + 1], xg2[q]);
+                    vF[c + 1] = f2_fma(w2[q], gF[q][c + 1], vF[c + 1]);
                 }
+            }
+#pragma unroll
+            for (int q = 0; q < PX; ++q) {
                 float xlo, xhi;
-                f2_split(xg2, xlo, xhi);
+                f2_split(xg2[q], xlo, xhi);
                 const float xg = xlo + xhi;  // dL/d(blended value) . (c, z, f) of this Gaussian
                 // dL/dalpha where alpha is not clamped, 0 elsewhere
-                const float dal = use[q] && alpha[q] < bp.alpha_max ? T[q] * xg - acc[q] * rom : 0.f;
-                acc[q] = fmaf(w, xg, acc[q]);
+                const float dal = use[q] && alpha[q] < bp.alpha_max ? T[q] * xg - acc[q] * rom[q] : 0.f;
+                acc[q] = fmaf(w[q], xg, acc[q]);
                 const float t = dal * G[q];
                 sop += t;
                 const float ty = t * dy[q];
                 sty += ty;
                 styy = fmaf(ty, dy[q], styy);
-                sca = f2_fma(w2, gCa[q], sca);
-                scb = f2_fma(w2, gCb[q], scb);
             }
             // record groups: du dv dz do | dca dcb dcc - | dr dg db - | df...
             float4 v[NG];
