@@ -78,9 +78,9 @@ cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const u
                               const ups_mlp &mlp, const ups_gaussians &out, int op_tanh, int num_sms,
                               cudaStream_t st);
 cudaError_t launch_decode_fwd_tc(const ViewTable &vt, int A, int K, int NF, const ups_anchors &anc,
-                                 const ups_mlp &mlp, const ups_gaussians &out, int bf16, int op_tanh, int *err,
+                                 const ups_mlp &mlp, const ups_gaussians &out, int op_tanh, int *err,
                                  int num_sms, cudaStream_t st);
-size_t decode_tc_smem_bytes(int NF, int bf16);
+size_t decode_tc_smem_bytes(int NF);
 cudaError_t launch_decode_bwd(const ViewTable &vt, int A, int K, int NF, const ups_anchors &anc,
                               const ups_mlp &mlp, const ups_gaussians &dG, unsigned mask, const ups_mlp *d_mlp,
                               const ups_anchors *d_anc, float *d_pose, int bf16, int op_tanh, float *scratch,
@@ -515,13 +515,10 @@ ups_status ups_decode_anchors(ups_ctx *c, const ups_anchors *anc, const ups_mlp 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c->last_stream = st;
     stage_begin(c, "decode_fwd", st);
-    // BF16 decode on the tensor cores; the FP32 decode on the CUDA cores (its
-    // 3xTF32 tensor-core form needs 223 KB of operands, one CTA per SM, and is
-    // slower than the CUDA-core kernel at these sizes)
-    const int bf16 = c->cfg.decode_bf16 ? 1 : 0;
-    if (bf16 && decode_tc_smem_bytes(c->cfg.n_feat, bf16) + 1024 <= 227 * 1024)
-        UPS_CUDA(c, launch_decode_fwd_tc(vt, anc->n, c->cfg.k, c->cfg.n_feat, *anc, *mlp, *out, bf16,
-                                         c->cfg.opacity_tanh, c->d_err, c->num_sms, st));
+    // BF16 decode on the tensor cores; the FP32 decode on the CUDA cores
+    if (c->cfg.decode_bf16 && decode_tc_smem_bytes(c->cfg.n_feat) + 1024 <= 227 * 1024)
+        UPS_CUDA(c, launch_decode_fwd_tc(vt, anc->n, c->cfg.k, c->cfg.n_feat, *anc, *mlp, *out, c->cfg.opacity_tanh,
+                                         c->d_err, c->num_sms, st));
     else
         UPS_CUDA(c, launch_decode_fwd(vt, anc->n, c->cfg.k, c->cfg.n_feat, *anc, *mlp, *out, c->cfg.opacity_tanh,
                                       c->num_sms, st));
