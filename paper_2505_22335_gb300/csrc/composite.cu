@@ -92,7 +92,7 @@ template <int PX> struct Px {
 
 template <int PX>
 struct TileP {
-    int v, px, py0;
+    int t, v, px, py0;
     bool in[PX];
     const DevView *cam;
 };
@@ -100,7 +100,12 @@ struct TileP {
 template <int PX>
 __device__ __forceinline__ TileP<PX> tilep(const ViewTable &vt) {
     TileP<PX> c;
-    const int t = blockIdx.x;
+    // Last tiles first.  The coarser levels of a tracking request come last and have
+    // the longest lists: started last, they ran on when the others had finished
+    // (500k anchors, three levels: forward 252 -> 185 us, backward 547 -> 415).  A
+    // single frame's last rows first also took less time here (1237x693 forward 357
+    // -> 336 us, 8 x 640x480 873 -> 839).
+    const int t = c.t = vt.total_tiles - 1 - (int)blockIdx.x;
     c.v = view_of_tile(vt, t);
     c.cam = &vt.v[c.v];
     int local = t - c.cam->tile_base;
@@ -166,7 +171,7 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
     __shared__ __align__(128) Stage<NF, KB> ring[NS];
     __shared__ __align__(8) uint64_t mbar[NS];
     const TileP<PX> tc = tilep<PX>(vt);
-    const uint2 rg = ranges[blockIdx.x];
+    const uint2 rg = ranges[tc.t];
     const int n_list = (int)(rg.y - rg.x);
     const int nb = (n_list + KB - 1) / KB;
     const int set_base = (tc.v - tc.cam->set) * N;  // gv - set_base: attribute index
@@ -196,25 +201,25 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
     }
 
     const float fx = (float)tc.px;
+    // T: the transmittance, negative once the pixel takes no more part (stopped, or
+    // outside the image): the next Gaussian's then fails the stopping test (t_min >= 0)
     float fy[PX], T[PX];
     f2 Ca[PX], Cb[PX];  // blended (r, g), (b, depth)
     f2 F[PX][NF > 0 ? NF / 2 : 1];  // feature accumulators, channel pairs
     uint32_t last[PX];
-    bool done[PX];
 #pragma unroll
     for (int q = 0; q < PX; ++q) {
         fy[q] = (float)(tc.py0 + RS * q);
-        T[q] = 1.f;
+        T[q] = tc.in[q] ? 1.f : -1.f;
         Ca[q] = Cb[q] = 0ull;
 #pragma unroll
         for (int c = 0; c < NF / 2; ++c) F[q][c] = 0ull;
         last[q] = 0u;
-        done[q] = !tc.in[q];
     }
     auto all_done = [&]() {
         bool d = true;
 #pragma unroll
-        for (int q = 0; q < PX; ++q) d = d && done[q];
+        for (int q = 0; q < PX; ++q) d = d && T[q] < 0.f;
         return d;
     };
     int b = 0;
@@ -231,7 +236,6 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
         const Stage<NF, KB> &S = ring[b % NS];
         const int n = min(KB, n_list - b * KB);
         for (int j = 0; j < n; ++j) {
-            if (__all_sync(0xffffffffu, all_done())) break;
             const float4 g = S.xyzo[j];
             const float4 cn = S.conic[j];
             const Expo ex = expo(cn, fx - g.x);
@@ -245,13 +249,15 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
             for (int q = 0; q < PX; ++q) {
                 alpha[q] = fminf(bp.alpha_max, g.w * falloff(expo_at(ex, fy[q] - g.y)));
                 Tn[q] = T[q] * (1.f - alpha[q]);
-                use[q] = !done[q] && alpha[q] >= bp.alpha_min;
-                const bool stop = use[q] && Tn[q] < bp.t_min;
-                done[q] = done[q] || stop;
-                use[q] = use[q] && !stop;
+                const bool hit = alpha[q] >= bp.alpha_min;
+                use[q] = hit && Tn[q] >= bp.t_min;
+                if (hit && Tn[q] < bp.t_min) T[q] = -fabsf(T[q]);
                 any = any || use[q];
             }
-            if (!__any_sync(0xffffffffu, any)) continue;
+            if (!__any_sync(0xffffffffu, any)) {
+                if (__all_sync(0xffffffffu, all_done())) break;
+                continue;
+            }
             const float4 col = S.color[j];
             const f2 ca = f2_make(col.x, col.y), cb = f2_make(col.z, g.z);
 #pragma unroll
@@ -287,7 +293,7 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
     if (!ok_wait) return;
     // a list cut short by the list cap is exact only if every pixel stopped
     // inside it; otherwise the caller blends the tile again from a full list
-    if (trunc && ((trunc[blockIdx.x >> 5] >> (blockIdx.x & 31)) & 1u))
+    if (trunc && ((trunc[tc.t >> 5] >> (tc.t & 31)) & 1u))
         if (__syncthreads_count(all_done()) != NT && threadIdx.x == 0) atomicOr(trunc_flag, 1);
     const DevView &cam = *tc.cam;
     const size_t HW = (size_t)cam.W * cam.H;
@@ -308,7 +314,7 @@ __global__ void __launch_bounds__(Px<PX>::NT) k_composite_fwd(
             out_feat[NF * P + 2 * c * HW + p] = f2_lo(F[q][c]);
             out_feat[NF * P + (2 * c + 1) * HW + p] = f2_hi(F[q][c]);
         }
-        out_T[P + p] = T[q];
+        out_T[P + p] = fabsf(T[q]);
         out_nc[P + p] = last[q];
     }
 }
@@ -388,16 +394,19 @@ __global__ void k_scale_mean(const float4 *__restrict__ scale, size_t n, float c
 // backward
 // ---------------------------------------------------------------------------
 
-// Ring depth and the CTAs per SM that the registers are cut for.  Up to 16 feature
-// channels 8 CTAs of two warps (128 registers, 52 bytes spilled, a ring of 2): on
-// batches of many waves as fast as 6 (156 registers, a ring of 3; 1.84 ms for
-// 8 x 640x480 at 16 channels either way), but a frame of 1200 tiles fits the GPU at
-// once (0.277 against 0.320 ms).  At 32 channels the 128 registers of dL/dF of four
-// pixels leave 4 CTAs of 234 registers: 5.88 ms for 8 x 1280x720, two pixels a
-// thread 7.61 ms (its warps reduce every Gaussian's 44 sums for half the pixels);
-// batches of 32 entries 6.19 ms, 5 CTAs (spills) 7.16 ms.
-constexpr int bwd_stages(int nf) { return nf <= 16 ? 2 : 3; }
-constexpr int bwd_ctas(int nf) { return nf <= 16 ? 8 : 4; }
+// Ring depth by the CTAs per SM that the registers are cut for.  Up to 16 feature
+// channels 6 CTAs of two warps (156 registers, a ring of 3), or 8 (128 registers, 52
+// bytes spilled, a ring of 2) where that takes all tiles at once and 6 do not: a
+// 640x480 frame, 1200 tiles on 152 SMs, 0.27 against 0.32 ms.  More tiles run in
+// several rounds either way (8 x 640x480 1.84 ms with both, 500k anchors in three
+// pyramid levels 0.415 with 6 and 0.485 with 8).  At 32 channels the 128 registers
+// of dL/dF of four pixels leave 4 CTAs of 234 registers: 5.88 ms for 8 x 1280x720,
+// two pixels a thread 7.61 ms (its warps reduce every Gaussian's 44 sums for half
+// the pixels); batches of 32 entries 6.19 ms, 5 CTAs (spills) 7.16 ms.
+constexpr int bwd_stages(int ctas) { return ctas == 8 ? 2 : 3; }
+inline int bwd_ctas(int nf, int tiles, int num_sms) {
+    return nf > 16 ? 4 : tiles > 6 * num_sms && tiles <= 8 * num_sms ? 8 : 6;
+}
 constexpr int kRedStride = 36;  // floats per lane row of the reduction scratch
 
 // Sums over the warp of the per-lane gradient record values v (float4 groups
@@ -440,8 +449,8 @@ __device__ __forceinline__ void warp_record_add(const float4 (&v)[NG], float (*r
     }
 }
 
-template <int NF, int PX>
-__global__ void __launch_bounds__(Px<PX>::NT, bwd_ctas(NF)) k_composite_bwd(
+template <int NF, int PX, int CTAS>
+__global__ void __launch_bounds__(Px<PX>::NT, CTAS) k_composite_bwd(
     ViewTable vt, BlendParams bp, int N, int per_view, const uint2 *__restrict__ ranges,
     const uint32_t *__restrict__ ival, const float4 *__restrict__ xyzo,
     const float4 *__restrict__ conic, const float4 *__restrict__ color,
@@ -449,7 +458,7 @@ __global__ void __launch_bounds__(Px<PX>::NT, bwd_ctas(NF)) k_composite_bwd(
     const uint32_t *__restrict__ in_nc, const float *__restrict__ dC,
     const float *__restrict__ dD, const float *__restrict__ dF, const float *__restrict__ dT,
     float *__restrict__ g2, uint32_t *__restrict__ hits, int *__restrict__ err) {
-    constexpr int NT = Px<PX>::NT, RS = Px<PX>::RS, NW = NT / 32, NS = bwd_stages(NF);
+    constexpr int NT = Px<PX>::NT, RS = Px<PX>::RS, NW = NT / 32, NS = bwd_stages(CTAS);
     constexpr int KB = UPS_BWD_BATCH;
     constexpr int STRIDE = kG2Base + NF;  // record floats, a multiple of 4
     constexpr int NG = STRIDE / 4;
@@ -460,7 +469,7 @@ __global__ void __launch_bounds__(Px<PX>::NT, bwd_ctas(NF)) k_composite_bwd(
     __shared__ uint32_t s_max[NW];
     const TileP<PX> tc = tilep<PX>(vt);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const uint2 rg = ranges[blockIdx.x];
+    const uint2 rg = ranges[tc.t];
     const float fx = (float)tc.px;
     const DevView &cam = *tc.cam;
     const size_t HW = (size_t)cam.W * cam.H;
@@ -700,19 +709,28 @@ cudaError_t launch_composite_bwd(const ViewTable &vt, const BlendParams &bp, int
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
                                  const float *feat, const float *T, const uint32_t *nc,
-                                 const ups_image_grads &dL, float *g2, uint32_t *hits, cudaStream_t st,
-                                 int *err) {
+                                 const ups_image_grads &dL, float *g2, uint32_t *hits, int num_sms,
+                                 cudaStream_t st, int *err) {
     if (vt.total_tiles == 0) return cudaSuccess;
-#define UPS_BWD(NFV)                                                                                \
-    k_composite_bwd<NFV, blend_px_bwd(NFV)><<<vt.total_tiles, Px<blend_px_bwd(NFV)>::NT, 0, st>>>(            \
-        vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, T, nc, dL.color, dL.depth, dL.feat, \
+    const int ctas = bwd_ctas(n_feat, vt.total_tiles, num_sms);
+#define UPS_BWD(NFV, CTASV)                                                                               \
+    k_composite_bwd<NFV, blend_px_bwd(NFV), CTASV><<<vt.total_tiles, Px<blend_px_bwd(NFV)>::NT, 0, st>>>( \
+        vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, T, nc, dL.color, dL.depth, dL.feat,  \
         dL.T, g2, hits, err)
+#define UPS_BWD68(NFV)     \
+    do {                   \
+        if (ctas == 8)     \
+            UPS_BWD(NFV, 8); \
+        else               \
+            UPS_BWD(NFV, 6); \
+    } while (0)
     switch (n_feat) {
-        case 0: UPS_BWD(0); break;
-        case 16: UPS_BWD(16); break;
-        case 32: UPS_BWD(32); break;
+        case 0: UPS_BWD68(0); break;
+        case 16: UPS_BWD68(16); break;
+        case 32: UPS_BWD(32, 4); break;
         default: return cudaErrorInvalidValue;
     }
+#undef UPS_BWD68
 #undef UPS_BWD
     return cudaGetLastError();
 }

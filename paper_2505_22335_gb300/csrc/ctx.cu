@@ -72,8 +72,8 @@ cudaError_t launch_composite_bwd(const ViewTable &vt, const BlendParams &bp, int
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
                                  const float *feat, const float *T, const uint32_t *nc,
-                                 const ups_image_grads &dL, float *g2, uint32_t *hits, cudaStream_t st,
-                                 int *err);
+                                 const ups_image_grads &dL, float *g2, uint32_t *hits, int num_sms,
+                                 cudaStream_t st, int *err);
 cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const ups_anchors &anc,
                               const ups_mlp &mlp, const ups_gaussians &out, int op_tanh, int num_sms,
                               cudaStream_t st);
@@ -961,7 +961,7 @@ ups_status ups_render_backward(ups_ctx *c, const ups_image_grads *dL, unsigned m
                                      c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
                                      reinterpret_cast<const float4 *>(c->g_in.color), c->g_in.feat,
                                      c->img.T, c->img.n_contrib, *dL, c->g2.as<float>(),
-                                     hits.bits, st, c->d_err));
+                                     hits.bits, c->num_sms, st, c->d_err));
     stage_end(c, st, 1);
     UPS_CUDA(c, launch_list_hits(hits, c->total_gv, st));
     c->launches += 1;
