@@ -547,6 +547,9 @@ ups_status ups_submit(ups_server *srv, const ups_request *req, uint64_t *ticket)
  * released), UPS_PENDING while queued or running, UPS_ERR_ARG for an unknown
  * ticket. */
 ups_status ups_poll(ups_server *srv, uint64_t ticket, ups_result *out);
+/* As ups_poll, but blocks until the request is done, at most timeout_ms
+ * (UPS_PENDING then). */
+ups_status ups_wait(ups_server *srv, uint64_t ticket, double timeout_ms, ups_result *out);
 /* Removes a request that has not started: UPS_OK (its poll then reports
  * UPS_ERR_CANCELLED), UPS_ERR_STATE if it already started. */
 ups_status ups_cancel(ups_server *srv, uint64_t ticket);

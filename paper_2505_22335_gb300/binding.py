@@ -117,7 +117,7 @@ EXPORTS = ["ups_config_default", "ups_version", "ups_create", "ups_destroy", "up
            "ups_anchor_update",
            "ups_render_backward", "ups_decode_backward", "ups_get_stats", "ups_copy_buffer",
            "ups_profile_enable", "ups_profile_read", "ups_render_forward_static",
-           "ups_server_create", "ups_server_destroy", "ups_submit", "ups_poll", "ups_cancel",
+           "ups_server_create", "ups_server_destroy", "ups_submit", "ups_poll", "ups_wait", "ups_cancel",
            "ups_server_wait_idle", "ups_server_set_scene", "ups_server_last_error"]
 
 _lib = None
@@ -175,6 +175,7 @@ def load():
     L.ups_server_destroy.argtypes = [_p]
     L.ups_submit.argtypes = [_p, C.POINTER(Request), C.POINTER(C.c_uint64)]
     L.ups_poll.argtypes = [_p, C.c_uint64, C.POINTER(Result)]
+    L.ups_wait.argtypes = [_p, C.c_uint64, C.c_double, C.POINTER(Result)]
     L.ups_cancel.argtypes = [_p, C.c_uint64]
     L.ups_server_wait_idle.argtypes = [_p, C.c_double]
     L.ups_server_set_scene.argtypes = [_p, C.POINTER(Anchors), C.POINTER(MLP), C.c_double]
@@ -563,7 +564,9 @@ class Server:
     def poll(self, ticket):
         """-> None while pending, else a dict (status, times in ms, batch info)."""
         r = Result()
-        st = self._L.ups_poll(self._h, ticket, C.byref(r))
+        return self._result(ticket, self._L.ups_poll(self._h, ticket, C.byref(r)), r)
+
+    def _result(self, ticket, st, r):
         if st == UPS_PENDING:
             return None
         if st != UPS_OK:
@@ -578,12 +581,14 @@ class Server:
         import time
         t_end = time.time() + timeout_s
         while True:
-            res = self.poll(ticket)
+            # in slices, so that an interrupt of the interpreter is seen
+            left = max(0.0, min(0.2, t_end - time.time()))
+            r = Result()
+            res = self._result(ticket, self._L.ups_wait(self._h, ticket, left * 1e3, C.byref(r)), r)
             if res is not None:
                 return res
             if time.time() > t_end:
                 raise UpsError(5, "request did not finish in time")
-            time.sleep(0.0005)
 
     def wait_idle(self, timeout_s=120.0):
         st = self._L.ups_server_wait_idle(self._h, timeout_s * 1e3)

@@ -102,6 +102,7 @@ struct ups_server {
     int next_batch = 0;
     size_t reserved = 0, budget = 0;
     int in_flight = 0;
+    int waiters = 0;  // calls inside ups_wait
     std::chrono::steady_clock::time_point t0;
     std::string err;
     double now_ms() const {
@@ -269,6 +270,7 @@ void worker(ups_server *s, int si) {
                     r->started = true;
                     r->status = UPS_ERR_STATE;
                     r->t_start = r->t_end = s->now_ms();
+                    s->cv.notify_all();
                     s->err = "mapping request with anchor gradients submitted for a scene of " +
                              std::to_string(r->anc_n) + " anchors, scene now has " + std::to_string(s->anc.n);
                     continue;
@@ -371,9 +373,9 @@ ups_status ups_server_destroy(ups_server *s) {
     cudaSetDevice(s->device);
     for (Slot &sl : s->slots) cudaStreamSynchronize(sl.st);
     {
-        // host callbacks of the last batches
+        // host callbacks of the last batches, and callers of ups_wait
         std::unique_lock<std::mutex> lk(s->mu);
-        s->cv.wait_for(lk, std::chrono::seconds(30), [&] { return s->in_flight == 0; });
+        s->cv.wait_for(lk, std::chrono::seconds(30), [&] { return s->in_flight == 0 && s->waiters == 0; });
     }
     for (Slot &sl : s->slots) {
         for (Buf &b : sl.g) b.release();
@@ -440,9 +442,8 @@ ups_status ups_submit(ups_server *s, const ups_request *req, uint64_t *ticket) {
     return UPS_OK;
 }
 
-ups_status ups_poll(ups_server *s, uint64_t ticket, ups_result *out) {
-    if (!s) return UPS_ERR_ARG;
-    std::lock_guard<std::mutex> lk(s->mu);
+// the result of a request and, once it is done, the end of its entry (s->mu held)
+static ups_status take_result(ups_server *s, uint64_t ticket, ups_result *out) {
     auto it = s->reqs.find(ticket);
     if (it == s->reqs.end()) return UPS_ERR_ARG;
     Req *r = it->second;
@@ -461,6 +462,28 @@ ups_status ups_poll(ups_server *s, uint64_t ticket, ups_result *out) {
     return UPS_OK;
 }
 
+ups_status ups_poll(ups_server *s, uint64_t ticket, ups_result *out) {
+    if (!s) return UPS_ERR_ARG;
+    std::lock_guard<std::mutex> lk(s->mu);
+    return take_result(s, ticket, out);
+}
+
+// Woken by the end of a batch: a caller that polled every half millisecond saw a
+// tracking request of 3 ms a quarter of a millisecond late on average.
+ups_status ups_wait(ups_server *s, uint64_t ticket, double timeout_ms, ups_result *out) {
+    if (!s) return UPS_ERR_ARG;
+    std::unique_lock<std::mutex> lk(s->mu);
+    s->waiters++;
+    s->cv.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms), [&] {
+        auto it = s->reqs.find(ticket);
+        return it == s->reqs.end() || it->second->status != UPS_PENDING;
+    });
+    const ups_status st = take_result(s, ticket, out);
+    // the last use of the server: ups_server_destroy waits for it
+    if (--s->waiters == 0) s->cv.notify_all();
+    return st;
+}
+
 ups_status ups_cancel(ups_server *s, uint64_t ticket) {
     if (!s) return UPS_ERR_ARG;
     std::lock_guard<std::mutex> lk(s->mu);
@@ -471,6 +494,7 @@ ups_status ups_cancel(ups_server *s, uint64_t ticket) {
     s->queue.erase(std::remove(s->queue.begin(), s->queue.end(), r), s->queue.end());
     r->status = UPS_ERR_CANCELLED;
     r->t_end = s->now_ms();
+    s->cv.notify_all();
     return UPS_OK;
 }
 
