@@ -163,6 +163,24 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
             e0[i] = f2_fma(neg, c0[i], at(1));
             e2[i] = f2_fma(neg, c2[i], at(3));
         }
+        // Pass 2 steps the pre-activation along x, which rounds it another way than the
+        // corner-by-corner sum of pass 1 (both within 14 roundings of the magnitudes
+        // summed, 2^-20 of their sum): where a unit is nearer to 0 than that, pass 2
+        // takes pass 1's sum, so that both take the same units for on.
+        float near0 = 0.f;
+        {
+            const float4 b = reinterpret_cast<const float4 *>(s_b1)[lane];
+            float m[4] = {fabsf(b.x), fabsf(b.y), fabsf(b.z), fabsf(b.w)};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float4 z = reinterpret_cast<const float4 *>(s_z[w][c])[lane];
+                m[0] += fabsf(z.x);
+                m[1] += fabsf(z.y);
+                m[2] += fabsf(z.z);
+                m[3] += fabsf(z.w);
+            }
+            near0 = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])) * 9.5367431640625e-7f;
+        }
         f2 aD[4][2] = {};
         // units of at most kUnit pixels: bw columns, br rows
         for (int bx = xs; bx < xe; bx += kUnit) {
@@ -241,10 +259,24 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                     for (int x = 0; x < bw; ++x) {
                         const float2 t = px[x];
                         const f2 ax2 = f2_make(t.y, t.y);
-                        const f2 za = f2_fma(ax2, sla, z0a), zb = f2_fma(ax2, slb, z0b);
+                        f2 za = f2_fma(ax2, sla, z0a), zb = f2_fma(ax2, slb, z0b);
                         float u0, u1, u2, u3;
                         f2_split(za, u0, u1);
                         f2_split(zb, u2, u3);
+                        if (fminf(fminf(fabsf(u0), fabsf(u1)), fminf(fabsf(u2), fabsf(u3))) <= near0) {
+                            const float wt[4] = {(1.f - t.y) * (1.f - ay), t.y * (1.f - ay), (1.f - t.y) * ay, t.y * ay};
+                            za = bb01;
+                            zb = bb23;
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const ulonglong2 zc = reinterpret_cast<const ulonglong2 *>(s_z[w][c])[lane];
+                                const f2 w2c = f2_make(wt[c], wt[c]);
+                                za = f2_fma(w2c, zc.x, za);
+                                zb = f2_fma(w2c, zc.y, zb);
+                            }
+                            f2_split(za, u0, u1);
+                            f2_split(zb, u2, u3);
+                        }
                         const f2 ma = f2_make(u0 > 0.f ? t.x : 0.f, u1 > 0.f ? t.x : 0.f);
                         const f2 mb = f2_make(u2 > 0.f ? t.x : 0.f, u3 > 0.f ? t.x : 0.f);
                         S0a = f2_add(S0a, ma);
