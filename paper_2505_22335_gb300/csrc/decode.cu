@@ -532,13 +532,33 @@ __device__ __forceinline__ void bwd_group(const dbwd::Args &a, const DecodeArgs 
     }
 }
 
-// One thread per row (anchor-major), 128 rows per step of a grid-stride loop;
+// One thread per row (anchor-major), kRowsFp32 rows per step of a grid-stride loop;
 // weights in shared memory read as broadcasts.
-template <int NF>
+//
+// A row's chain through its four MLPs takes about 0.12 ms however few rows there
+// are.  Few rows (at most max_split_tiles CTAs' worth, half of what the GPU holds)
+// are therefore split by MLP: CTA (x, y) does one MLP of its rows, and as the end of
+// a row's backward is linear in dL/dx, every MLP's share goes through it by itself
+// (the Gaussians' means with the opacity MLP, the anchor scaling with the
+// covariance).  10k rows 0.126 -> 0.086 ms; a tracking request over 500k anchors,
+// whose list of rows is short, 2.91 -> 2.82.  More rows than that fill the GPU as
+// they are, and the four ends would cost them (SPLIT false: no such choice, and
+// fewer registers spilled).
+template <int NF, bool SPLIT>
 __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decode_bwd_rows(ViewTable vt,
-                                                                                               dbwd::Args a) {
+                                                                                               dbwd::Args a,
+                                                                                               int max_split_tiles) {
     extern __shared__ float4 smem4[];
     __shared__ float aPose[3 * UPS_MAX_VIEWS];
+    const int end = a.rows ? (int)*a.n_rows : a.row_end;
+    const int step = (int)gridDim.x * dbwd::kRowsFp32;
+    const bool split = SPLIT && (end - a.row_begin + dbwd::kRowsFp32 - 1) / dbwd::kRowsFp32 <= max_split_tiles;
+    if (!split && blockIdx.y) return;
+    // the MLP of this CTA, the costliest first (-1: all)
+    constexpr int kFirst = NF > 0 ? 0 : 1;
+    const int y = (int)blockIdx.y + kFirst;
+    const int only = !split ? -1 : y == 0 ? 3 : y == 1 ? 1 : y == 2 ? 2 : 0;
+    auto does = [&](int g) { return !SPLIT || only < 0 || only == g; };
     float *sm = reinterpret_cast<float *>(smem4);
     const int n_out = dbwd::n_out(a.K, NF);
     const DecodeArgs da{a.A, a.K, NF, n_out, a.pos, a.afeat, a.offs, a.ascale, a.w1, a.b1, a.w2, a.b2, a.op_tanh};
@@ -552,8 +572,7 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
     __syncthreads();
     const size_t NG = (size_t)a.A * a.K;
     float *sDX = sDXall + threadIdx.x;
-    const int end = a.rows ? (int)*a.n_rows : a.row_end;
-    for (int base = a.row_begin + blockIdx.x * dbwd::kRowsFp32; base < end; base += gridDim.x * dbwd::kRowsFp32) {
+    for (int base = a.row_begin + blockIdx.x * dbwd::kRowsFp32; base < end; base += step) {
         const bool valid = base + (int)threadIdx.x < end;
         const int row = a.rows && valid ? (int)a.rows[base + threadIdx.x] : base + (int)threadIdx.x;
         const int an = valid ? row / V : 0, v = valid ? row - an * V : 0;
@@ -562,7 +581,7 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
         const size_t gbase = (size_t)v * NG + (size_t)an * a.K;
         float x[kDinP], delta[3], dist;
         mlp_input(da, cam, an, x, delta, dist);
-        if (a.s.X && valid) {
+        if (a.s.X && valid && does(1)) {
             x[38] = 1.f;
 #pragma unroll
             for (int i = 0; i < kDinP; ++i) a.s.X[(size_t)i * a.s.ld + lr] = x[i];
@@ -571,14 +590,14 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
 #pragma unroll
         for (int i = 0; i < kDX; ++i) sDX[i * dbwd::kRowsFp32] = 0.f;
         float dls[3] = {0.f, 0.f, 0.f};
-        bwd_group<0, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
-        bwd_group<1, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
-        bwd_group<2, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
-        if (NF > 0) bwd_group<3, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
+        if (does(0)) bwd_group<0, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
+        if (does(1)) bwd_group<1, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
+        if (does(2)) bwd_group<2, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
+        if (NF > 0 && does(3)) bwd_group<3, NF>(a, da, sW1T, sb1, sW2, sb2, xt, an, valid, gbase, lr, sDX, dls);
         float dx[kDX];
 #pragma unroll
         for (int i = 0; i < kDX; ++i) dx[i] = sDX[i * dbwd::kRowsFp32];
-        dbwd::row_epilogue(a, valid ? an : -1, v, gbase, dx, delta, dist, dls, aPose);
+        dbwd::row_epilogue(a, valid ? an : -1, v, gbase, dx, delta, dist, dls, aPose, does(0), does(1));
     }
     __syncthreads();
     dbwd::flush_pose(a, vt, aPose);
@@ -652,13 +671,24 @@ cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a
     const size_t smem = bwd_rows_smem(dbwd::n_out(a.K, a.NF));
     if (smem > kMaxSmem) return cudaErrorInvalidConfiguration;
     const int rows = a.row_end - a.row_begin;
-    const int blocks = std::max(
-        1, std::min((rows + dbwd::kRowsFp32 - 1) / dbwd::kRowsFp32, num_sms * dbwd::kRowsCtasPerSm));
-#define UPS_DECB(NFV)                                                                              \
-    do {                                                                                           \
-        cudaFuncSetAttribute(k_decode_bwd_rows<NFV>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
-                             (int)smem);                                                           \
-        k_decode_bwd_rows<NFV><<<blocks, dbwd::kRowsFp32, smem, st>>>(vt, a);                  \
+    const int tiles = (rows + dbwd::kRowsFp32 - 1) / dbwd::kRowsFp32;
+    const int blocks = std::max(1, std::min(tiles, num_sms * dbwd::kRowsCtasPerSm));
+    // (of a list, whose length only the GPU knows, the kernel decides)
+    const int max_split = num_sms * dbwd::kRowsCtasPerSm / 2;
+    const bool split = a.rows || tiles <= max_split;
+    const dim3 grid(blocks, split ? (a.NF > 0 ? 4 : 3) : 1);
+#define UPS_DECB1(NFV, SPLITV)                                                                            \
+    do {                                                                                                  \
+        cudaFuncSetAttribute(k_decode_bwd_rows<NFV, SPLITV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                             (int)smem);                                                                  \
+        k_decode_bwd_rows<NFV, SPLITV><<<grid, dbwd::kRowsFp32, smem, st>>>(vt, a, max_split);            \
+    } while (0)
+#define UPS_DECB(NFV)              \
+    do {                           \
+        if (split)                 \
+            UPS_DECB1(NFV, true);  \
+        else                       \
+            UPS_DECB1(NFV, false); \
     } while (0)
     switch (a.NF) {
         case 0: UPS_DECB(0); break;
@@ -667,6 +697,7 @@ cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a
         default: return cudaErrorInvalidValue;
     }
 #undef UPS_DECB
+#undef UPS_DECB1
     return cudaGetLastError();
 }
 

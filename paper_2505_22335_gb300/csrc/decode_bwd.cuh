@@ -145,15 +145,15 @@ __device__ __forceinline__ SegInfo seg_info(int an) {  // an < 0: invalid row
 // The end of a row's backward, all threads of the warp together (invalid
 // rows pass an = -1 and zeros):
 //   dx[0..31] = dL/df_v, dx[32..34] = dL/d delta_vc, dx[35] = dL/d d_vc;
-//   dls = dL/d(anchor scaling) of this row; the dL/d(mean) of the row's K
-//   Gaussians are read from d_mean_op.
+//   dls = dL/d(anchor scaling) of this row (added if `scaling`); the dL/d(mean) of
+//   the row's K Gaussians are read from d_mean_op (if `means`).
 // delta_vc = r / |r|, d_vc = |r| with r = x_v - o_c:  dL/dr = (I - delta
 // delta^T) dL/d delta / d + dL/dd delta; x_v gets +dL/dr and the camera centre
 // -dL/dr (accumulated per view in aPose, shared memory).  Anchor values are
 // summed over the anchor's rows in the warp: one atomic per anchor and value.
 __device__ __forceinline__ void row_epilogue(const Args &a, int an, int v, size_t gbase, const float dx[36],
                                              const float delta[3], float dist, const float dls[3],
-                                             float *aPose) {
+                                             float *aPose, bool means = true, bool scaling = true) {
     const bool valid = an >= 0;
     const SegInfo si = seg_info(an);
     float dr[3] = {0.f, 0.f, 0.f};
@@ -173,7 +173,7 @@ __device__ __forceinline__ void row_epilogue(const Args &a, int an, int v, size_
         if (si.tail) atomicAdd(a.g_afeat + (size_t)an * kFin + i, s);
     }
     float dpos[3] = {dr[0], dr[1], dr[2]};
-    for (int k = 0; k < a.K; ++k) {
+    for (int k = 0; k < (means ? a.K : 0); ++k) {
         const float4 dm = valid ? a.d_mean_op[gbase + k] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float d3[3] = {dm.x, dm.y, dm.z};
 #pragma unroll
@@ -186,10 +186,10 @@ __device__ __forceinline__ void row_epilogue(const Args &a, int an, int v, size_
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
         const float sp = seg_scan(dpos[c], si.ok);
-        const float sl = seg_scan(valid ? dls[c] : 0.f, si.ok);
-        if (si.tail) {
-            atomicAdd(a.g_pos + 3 * an + c, sp);
-            atomicAdd(a.g_ascale + 3 * an + c, sl);
+        if (si.tail) atomicAdd(a.g_pos + 3 * an + c, sp);
+        if (scaling) {
+            const float sl = seg_scan(valid ? dls[c] : 0.f, si.ok);
+            if (si.tail) atomicAdd(a.g_ascale + 3 * an + c, sl);
         }
     }
 }
