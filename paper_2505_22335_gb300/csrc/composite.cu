@@ -118,13 +118,15 @@ __device__ __forceinline__ TileP<PX> tilep(const ViewTable &vt) {
     return c;
 }
 
-// pixels per thread: forward 2; backward 4 (the per-Gaussian warp reduction is
-// shared by more pixels)
-#ifndef UPS_FWD_PX
-#define UPS_FWD_PX 2
-#endif
-__host__ __device__ constexpr int blend_px_fwd(int nf) { return UPS_FWD_PX; }
-__host__ __device__ constexpr int blend_px_bwd(int nf) { return 4; }
+// Pixels per thread: forward 2; backward 4 (the per-Gaussian warp reduction is
+// shared by more pixels).  Few tiles (at most two per SM) leave the SMs waiting for
+// one list entry after another: there half as many pixels a thread and twice the
+// warps a tile (backward, 16 channels: 80 tiles 0.403 -> 0.275 ms, 300 tiles 0.233 ->
+// 0.193; forward 0.157 -> 0.134 and 0.097 -> 0.087; no channels, 2,000 Gaussians,
+// 80 tiles 0.040 -> 0.034).  At 690 tiles the forward (0.121 -> 0.124 ms) and the
+// 32-channel backward (0.410 -> 0.432) lose by it.
+constexpr int kPxFwd = 2, kPxBwd = 4, kPxFwdSmall = 1, kPxBwdSmall = 2, kSmallCtas = 2;
+inline bool few_tiles(int tiles, int num_sms) { return tiles <= 2 * num_sms; }
 
 // Exponent coefficients of a staged Gaussian for a thread's pixel column, in
 // base 2: exp(p) = 2^(p log2 e), so the coefficients carry the factor log2 e
@@ -403,7 +405,7 @@ __global__ void k_scale_mean(const float4 *__restrict__ scale, size_t n, float c
 // of dL/dF of four pixels leave 4 CTAs of 234 registers: 5.88 ms for 8 x 1280x720,
 // two pixels a thread 7.61 ms (its warps reduce every Gaussian's 44 sums for half
 // the pixels); batches of 32 entries 6.19 ms, 5 CTAs (spills) 7.16 ms.
-constexpr int bwd_stages(int ctas) { return ctas == 8 ? 2 : 3; }
+constexpr int bwd_stages(int ctas) { return ctas == 8 || ctas == kSmallCtas ? 2 : 3; }
 inline int bwd_ctas(int nf, int tiles, int num_sms) {
     return nf > 16 ? 4 : tiles > 6 * num_sms && tiles <= 8 * num_sms ? 8 : 6;
 }
@@ -659,19 +661,28 @@ __global__ void __launch_bounds__(Px<PX>::NT, CTAS) k_composite_bwd(
 cudaError_t launch_composite_fwd(const ViewTable &vt, const BlendParams &bp, int n_feat, int N,
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
-                                 const float *feat, const ups_images &out, cudaStream_t st,
+                                 const float *feat, const ups_images &out, int num_sms, cudaStream_t st,
                                  const uint32_t *trunc, int *trunc_flag, const int *gate, int *err) {
     if (vt.total_tiles == 0) return cudaSuccess;
-#define UPS_FWD(NFV)                                                                                  \
-    k_composite_fwd<NFV, blend_px_fwd(NFV)><<<vt.total_tiles, Px<blend_px_fwd(NFV)>::NT, 0, st>>>(              \
-        vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, out.color, out.depth, out.feat, out.T, \
+    const bool small = few_tiles(vt.total_tiles, num_sms);
+#define UPS_FWD1(NFV, PXV)                                                                                       \
+    k_composite_fwd<NFV, PXV><<<vt.total_tiles, Px<PXV>::NT, 0, st>>>(                                           \
+        vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, out.color, out.depth, out.feat, out.T,      \
         out.n_contrib, trunc, trunc_flag, gate, err)
+#define UPS_FWD(NFV)                   \
+    do {                               \
+        if (small)                     \
+            UPS_FWD1(NFV, kPxFwdSmall); \
+        else                           \
+            UPS_FWD1(NFV, kPxFwd);     \
+    } while (0)
     switch (n_feat) {
         case 0: UPS_FWD(0); break;
         case 16: UPS_FWD(16); break;
         case 32: UPS_FWD(32); break;
         default: return cudaErrorInvalidValue;
     }
+#undef UPS_FWD1
 #undef UPS_FWD
     return cudaGetLastError();
 }
@@ -713,21 +724,29 @@ cudaError_t launch_composite_bwd(const ViewTable &vt, const BlendParams &bp, int
                                  cudaStream_t st, int *err) {
     if (vt.total_tiles == 0) return cudaSuccess;
     const int ctas = bwd_ctas(n_feat, vt.total_tiles, num_sms);
-#define UPS_BWD(NFV, CTASV)                                                                               \
-    k_composite_bwd<NFV, blend_px_bwd(NFV), CTASV><<<vt.total_tiles, Px<blend_px_bwd(NFV)>::NT, 0, st>>>( \
+    const bool small = few_tiles(vt.total_tiles, num_sms);
+#define UPS_BWD(NFV, PXV, CTASV)                                                                               \
+    k_composite_bwd<NFV, PXV, CTASV><<<vt.total_tiles, Px<PXV>::NT, 0, st>>>(                             \
         vt, bp, N, per_view, ranges, ival, xyzo, conic, color, feat, T, nc, dL.color, dL.depth, dL.feat,  \
         dL.T, g2, hits, err)
-#define UPS_BWD68(NFV)     \
-    do {                   \
-        if (ctas == 8)     \
-            UPS_BWD(NFV, 8); \
-        else               \
-            UPS_BWD(NFV, 6); \
+#define UPS_BWD68(NFV)                            \
+    do {                                          \
+        if (small)                                \
+            UPS_BWD(NFV, kPxBwdSmall, kSmallCtas); \
+        else if (ctas == 8)                       \
+            UPS_BWD(NFV, kPxBwd, 8);              \
+        else                                      \
+            UPS_BWD(NFV, kPxBwd, 6);              \
     } while (0)
     switch (n_feat) {
         case 0: UPS_BWD68(0); break;
         case 16: UPS_BWD68(16); break;
-        case 32: UPS_BWD(32, 4); break;
+        case 32:
+            if (small)
+                UPS_BWD(32, kPxBwdSmall, kSmallCtas);
+            else
+                UPS_BWD(32, kPxBwd, 4);
+            break;
         default: return cudaErrorInvalidValue;
     }
 #undef UPS_BWD68

@@ -37,7 +37,7 @@ cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N
 cudaError_t launch_composite_fwd(const ViewTable &vt, const BlendParams &bp, int n_feat, int N,
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
-                                 const float *feat, const ups_images &out, cudaStream_t st,
+                                 const float *feat, const ups_images &out, int num_sms, cudaStream_t st,
                                  const uint32_t *trunc = nullptr, int *trunc_flag = nullptr,
                                  const int *gate = nullptr, int *err = nullptr);
 size_t anchor_scratch_bytes(size_t n, size_t P);
@@ -675,7 +675,7 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     stage_begin(c, "composite_fwd", st);
     UPS_CUDA(c, launch_composite_fwd(vt, c->bp, c->cfg.n_feat, c->N, c->per_view, c->ranges.as<uint2>(),
                                      c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                                     reinterpret_cast<const float4 *>(g->color), g->feat, *out, st,
+                                     reinterpret_cast<const float4 *>(g->color), g->feat, *out, c->num_sms, st,
                                      capped ? c->trunc.as<uint32_t>() : nullptr, capped ? c->d_trunc_flag : nullptr,
                                      nullptr, c->d_err));
     stage_end(c, st, 1);
@@ -687,7 +687,7 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
         UPS_CUDA(c, lists(kNoListCap, c->d_trunc_flag));
         UPS_CUDA(c, launch_composite_fwd(vt, c->bp, c->cfg.n_feat, c->N, c->per_view, c->ranges.as<uint2>(),
                                          c->ival_sorted, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                                         reinterpret_cast<const float4 *>(g->color), g->feat, *out, st, nullptr,
+                                         reinterpret_cast<const float4 *>(g->color), g->feat, *out, c->num_sms, st, nullptr,
                                          nullptr, c->d_trunc_flag, c->d_err));
         stage_end(c, st, 3);
     }

@@ -45,7 +45,7 @@ cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaS
 cudaError_t launch_composite_fwd(const ViewTable &vt, const BlendParams &bp, int n_feat, int N,
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
-                                 const float *feat, const ups_images &out, cudaStream_t st,
+                                 const float *feat, const ups_images &out, int num_sms, cudaStream_t st,
                                  const uint32_t *trunc = nullptr, int *trunc_flag = nullptr,
                                  const int *gate = nullptr, int *err = nullptr);
 cudaError_t radix_sort_u32_fixed(uint32_t **key_io, uint32_t **key_alt, uint32_t **val_io,
@@ -225,6 +225,6 @@ extern "C" ups_status ups_render_forward_static(const ups_config *cfg, const ups
     NA_CUDA(cudaMemsetAsync(ranges, 0, (size_t)vt.total_tiles * sizeof(uint2), st));
     NA_CUDA(launch_ranges(ik, (uint32_t)n_inst, ranges, st));
     NA_CUDA(launch_composite_fwd(vt, bp, nf, N, per_view, ranges, iv, xyzo, conic,
-                                 reinterpret_cast<const float4 *>(g->color), g->feat, *out, st));
+                                 reinterpret_cast<const float4 *>(g->color), g->feat, *out, 0, st));
     return UPS_OK;
 }
