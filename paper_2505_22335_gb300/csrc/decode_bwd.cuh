@@ -224,8 +224,8 @@ cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a
 cudaError_t launch_live_rows(const dbwd::Args &a, int V, uint32_t *rows, uint32_t *n_rows, cudaStream_t st);
 cudaError_t launch_decode_bwd_rows_tc(const ViewTable &vt, const dbwd::Args &a, int num_sms, cudaStream_t st);
 size_t decode_bwd_rows_tc_smem(int NF, int K);
-// rows the per-row kernel's resident grid covers in one pass (FP32: 3 CTAs of
-// 128 rows per SM; tcgen05: 1 or 2 CTAs per SM by shared memory)
+// rows the per-row kernel's resident grid covers in one pass (FP32: 2 CTAs of
+// 256 rows per SM; tcgen05: 1 or 2 CTAs per SM by shared memory)
 int decode_bwd_rows_wave(int bf16, int K, int NF, int num_sms);
 bool decode_wgrad_tc_fits(int K, int NF);
 cudaError_t launch_decode_wgrad_tc(const float *scratch, int ld, int nrows, int K, int NF, const ups_mlp &d_mlp,
