@@ -517,11 +517,11 @@ Plan plan_of(const ViewTable &vt, int N, int num_sms) {
     return p;
 }
 
-// dynamic shared memory of a kernel (its static part counts against the default 48 KB too)
-cudaError_t allow_smem(const void *f, size_t bytes) {
-    return bytes > 40 * 1024 ? cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes)
-                             : cudaSuccess;
-}
+// The largest shared memory of a view: kMaxBinTiles tiles, at most kMaxSide a side
+// (16,384 pixels).
+constexpr int kMaxSide = 1024;
+constexpr FillShape kMaxFill{kMaxBinTiles, kMaxBinTiles / 32 + kMaxSide, kMaxBinTiles + 2 * kMaxSide + 1};
+constexpr size_t kMaxCountSmem = (size_t)(kMaxBinTiles + kMaxSide) * sizeof(int);
 
 }  // namespace
 
@@ -540,7 +540,7 @@ cudaError_t bin_count(const ViewTable &vt, float alpha_min, int N, const uint32_
                       const uint4 *more, const float4 *xyzo, const float4 *conic, void *scratch, int num_sms, cudaStream_t st) {
     const Plan p = plan_of(vt, N, num_sms);
     uint32_t *tot = static_cast<uint32_t *>(scratch), *cnt = tot + vt.total_tiles;
-    cudaError_t e = allow_smem((const void *)k_bin_count, p.count_smem);
+    cudaError_t e = allow_smem(k_bin_count, kMaxCountSmem);
     if (e != cudaSuccess) return e;
     k_bin_count<<<dim3(p.runs.nb, vt.n), kBinThreads, p.count_smem, st>>>(vt, alpha_min, p.runs, sorted_gv, span,
                                                                      more, xyzo, conic, cnt);
@@ -558,7 +558,7 @@ cudaError_t bin_lists(const ViewTable &vt, float alpha_min, int N, const uint32_
     const bool capped = cap != kNoListCap;
     const size_t smem = capped ? fill_smem<true>(p.fill) : fill_smem<false>(p.fill);
     const auto kernel = capped ? k_bin_fill<true> : k_bin_fill<false>;
-    const cudaError_t e = allow_smem((const void *)kernel, smem);
+    const cudaError_t e = allow_smem(kernel, capped ? fill_smem<true>(kMaxFill) : fill_smem<false>(kMaxFill));
     if (e != cudaSuccess) return e;
     kernel<<<dim3(vt.n, p.runs.nb), kBinThreads, smem, st>>>(vt, alpha_min, p.runs, sorted_gv, span, more, xyzo, conic,
                                                        cnt, tot, ranges, lists, gate);

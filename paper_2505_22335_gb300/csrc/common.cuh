@@ -96,6 +96,16 @@ __device__ __forceinline__ float f2_hi(f2 a) {
     return hi;
 }
 
+// Lets launches of a kernel ask for up to `most` bytes of dynamic shared memory.  The
+// limit belongs to the kernel on the device, not to the launch: threads launch the
+// same kernel with other sizes at the same time, so every caller sets one value that
+// no launch of the kernel exceeds, and never the size of its own.
+template <class F>
+inline cudaError_t allow_smem(F *kernel, size_t most) {
+    return cudaFuncSetAttribute(reinterpret_cast<const void *>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)most);
+}
+
 // Device buffer that only grows.
 struct DevBuf {
     void *ptr = nullptr;

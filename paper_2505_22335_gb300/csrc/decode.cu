@@ -679,8 +679,8 @@ cudaError_t launch_decode_bwd_rows_fp32(const ViewTable &vt, const dbwd::Args &a
     const dim3 grid(blocks, split ? (a.NF > 0 ? 4 : 3) : 1);
 #define UPS_DECB1(NFV, SPLITV)                                                                            \
     do {                                                                                                  \
-        cudaFuncSetAttribute(k_decode_bwd_rows<NFV, SPLITV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem);                                                                  \
+        const cudaError_t e = allow_smem(k_decode_bwd_rows<NFV, SPLITV>, bwd_rows_smem(dbwd::n_out(16, NFV))); \
+        if (e != cudaSuccess) return e;                                                                   \
         k_decode_bwd_rows<NFV, SPLITV><<<grid, dbwd::kRowsFp32, smem, st>>>(vt, a, max_split);            \
     } while (0)
 #define UPS_DECB(NFV)              \
@@ -726,8 +726,8 @@ cudaError_t launch_decode_fwd(const ViewTable &vt, int A, int K, int NF, const u
         pair = pair && reinterpret_cast<uintptr_t>(p) % 32 == 0;
 #define UPS_DEC1(NFV, PAIRV)                                                                       \
     do {                                                                                           \
-        cudaFuncSetAttribute(k_decode_fwd<NFV, PAIRV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem);                                                           \
+        const cudaError_t e = allow_smem(k_decode_fwd<NFV, PAIRV>, kMaxSmem);                      \
+        if (e != cudaSuccess) return e;                                                            \
         k_decode_fwd<NFV, PAIRV><<<blocks, 32 * warps, smem, st>>>(                                \
             vt, a, split, reinterpret_cast<float4 *>(out.mean_opacity),                            \
             reinterpret_cast<float4 *>(out.scale), reinterpret_cast<float4 *>(out.quat),           \

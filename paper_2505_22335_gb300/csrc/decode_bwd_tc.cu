@@ -661,7 +661,8 @@ cudaError_t launch_decode_wgrad(const WArgs &wa, int num_sms, cudaStream_t st) {
     const int blocks = std::max(1, std::min(chunks, num_sms));
 #define UPS_WG(U, T)                                                                                   \
     do {                                                                                               \
-        cudaFuncSetAttribute(k_decode_wgrad<U, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
+        const cudaError_t e = allow_smem(k_decode_wgrad<U, T>, 227 * 1024);                            \
+        if (e != cudaSuccess) return e;                                                                \
         k_decode_wgrad<U, T><<<blocks, T, smem, st>>>(wa, db);                                         \
     } while (0)
     if (n_mt <= 512 && w.fH <= 1024)
@@ -700,8 +701,8 @@ cudaError_t launch_decode_bwd_rows_tc(const ViewTable &vt, const dbwd::Args &a, 
     const int blocks = std::max(1, std::min((rows + kRows - 1) / kRows, num_sms * per_sm));
 #define UPS_BT(NFV)                                                                              \
     do {                                                                                         \
-        cudaFuncSetAttribute(k_decode_bwd_rows_tc<NFV>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                             (int)smem);                                                         \
+        const cudaError_t e = allow_smem(k_decode_bwd_rows_tc<NFV>, 226 * 1024);                 \
+        if (e != cudaSuccess) return e;                                                          \
         k_decode_bwd_rows_tc<NFV><<<blocks, kRows, smem, st>>>(vt, a);                           \
     } while (0)
     switch (a.NF) {

@@ -374,7 +374,8 @@ cudaError_t launch_decode_fwd_tc(const ViewTable &vt, int A, int K, int NF, cons
     const int blocks = std::max(1, std::min(tiles, num_sms * 2));
 #define UPS_TC(NFV)                                                                                               \
     do {                                                                                                          \
-        cudaFuncSetAttribute(k_decode_fwd_tc<NFV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);       \
+        const cudaError_t e = allow_smem(k_decode_fwd_tc<NFV>, decode_tc_smem_bytes(NFV));                        \
+        if (e != cudaSuccess) return e;                                                                           \
         k_decode_fwd_tc<NFV><<<blocks, kTCRows, smem, st>>>(vt, a);                                               \
     } while (0)
     switch (NF) {

@@ -1371,13 +1371,13 @@ cudaError_t lift_all(int num_sms, cudaStream_t st, const ViewTable &vt, int nf, 
         const size_t smem = lift_tc_smem_bytes();
         // one CTA per SM: it holds all 512 TMEM columns
         if (smem > 227 * 1024 || 2 * (smem + 1024) <= 228 * 1024) return cudaErrorInvalidConfiguration;
-        cudaFuncSetAttribute(k_lift_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if ((e = allow_smem(k_lift_tc, smem)) != cudaSuccess) return e;
         k_lift_tc<<<grid_ctas, lt::kAll, smem, st>>>(vt, np, patch, feat, w1, b1, M, E, sv, u, beta, gram, weight, g,
                                                    loss, D, alpha, sb, hb, Gb, d_w1, d_b1, d_feat, err);
     } else if (nf == 32) {
         // the BF16 operand tiles and the FP32 arrays of N_l = 32 exceed shared memory: all FP32 on the CUDA cores
         const size_t smem = fused_smem_bytes(nf);
-        cudaFuncSetAttribute(k_lift_fused<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if ((e = allow_smem(k_lift_fused<32>, smem)) != cudaSuccess) return e;
         k_lift_fused<32><<<grid_ctas, kFT, smem, st>>>(vt, np, patch, feat, w1, b1, M, E, sv, u, beta, gram, weight,
                                                        g, loss, D, alpha, sb, hb, Gb, d_w1, d_b1, d_feat);
     } else {

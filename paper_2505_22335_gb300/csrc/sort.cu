@@ -625,7 +625,7 @@ cudaError_t order_impl(K *key, K *key_alt, uint32_t *val, uint32_t *val_alt, siz
     if (passes > kOrderPasses || n > (size_t)INT32_MAX) return cudaErrorInvalidValue;
     if (n <= (size_t)kSmallOrder) {
         constexpr int smem = kSmallOrder * (sizeof(K) + 4) + kSmallWarps * kBins * 4;
-        const cudaError_t e = cudaFuncSetAttribute(k_order_small<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        const cudaError_t e = allow_smem(k_order_small<K>, smem);
         if (e != cudaSuccess) return e;
         k_order_small<K><<<1, kSmallThreads, smem, st>>>(key, (int)n, passes, val);
         *launches = 1;

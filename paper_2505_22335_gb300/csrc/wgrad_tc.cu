@@ -327,6 +327,20 @@ bool make_map(CUtensorMap *m, const float *scratch, int ld, int nrows, int nfeat
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+size_t wgrad_tc_smem(const WLay &w) { return (size_t)2 * w.set_bytes * w.stages + 1024; }
+
+// of every K and channel count that this kernel takes
+size_t wgrad_tc_most_smem() {
+    static const size_t most = [] {
+        size_t m = 0;
+        for (int NF : {0, 16, 32})
+            for (int K = 1; K <= 16; ++K)
+                if (const WLay w = wlay(K, NF); wlay_ok(w)) m = std::max(m, wgrad_tc_smem(w));
+        return m;
+    }();
+    return most;
+}
+
 }  // namespace
 
 bool decode_wgrad_tc_fits(int K, int NF) { return wlay_ok(wlay(K, NF)); }
@@ -345,11 +359,12 @@ cudaError_t launch_decode_wgrad_tc(const float *scratch, int ld, int nrows, int 
         !make_map(&maps.dy, scratch, ld, nrows, nfeat, kDyBox) ||
         !make_map(&maps.dy_last, scratch, ld, nrows, nfeat, w.wlast))
         return cudaErrorInvalidValue;
-    const size_t smem = (size_t)2 * w.set_bytes * w.stages + 1024;
+    const size_t smem = wgrad_tc_smem(w);
     WTArgs a{nrows, K, NF, d_mlp.w1, d_mlp.b1, d_mlp.w2, d_mlp.b2, err};
     const int chunks = (nrows + kKR - 1) / kKR;
     const int blocks = std::max(1, std::min(chunks, num_sms));
-    cudaFuncSetAttribute(k_decode_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_smem(k_decode_wgrad_tc, wgrad_tc_most_smem());
+    if (e != cudaSuccess) return e;
     k_decode_wgrad_tc<<<blocks, kT, smem, st>>>(maps, a);
     return cudaGetLastError();
 }
