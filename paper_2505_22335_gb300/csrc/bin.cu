@@ -33,6 +33,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "list_rules.cuh"
 #include "tiles.cuh"
 
 namespace ups {
@@ -66,7 +67,6 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(ViewTable vt, float a
     const int tx = cam.tiles_x, ty = cam.tiles_y, ld = tx + 1, lane = threadIdx.x & 31;
     for (int i = threadIdx.x; i < ld * ty; i += kBinThreads) diff[i] = 0;
     __syncthreads();
-    const uint32_t top = (uint32_t)runs.N * (uint32_t)vt.n - 1u;  // an order that lost a wait may hold any id
     const int beg = runs.beg(blockIdx.x), end = runs.end(blockIdx.x);
     const uint32_t *sg = sorted_gv + (size_t)blockIdx.y * runs.N;
     constexpr int U = 4;  // gathers in flight per thread
@@ -74,9 +74,10 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_count(ViewTable vt, float a
         uint32_t gv[U];
         uint4 s[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) gv[u] = i0 + u * kBinThreads < end ? min(sg[i0 + u * kBinThreads], top) : 0xffffffffu;
+        for (int u = 0; u < U; ++u) gv[u] = i0 + u * kBinThreads < end ? sg[i0 + u * kBinThreads] : 0xffffffffu;
 #pragma unroll
-        for (int u = 0; u < U; ++u) s[u] = gv[u] != 0xffffffffu ? span[gv[u]] : make_uint4(0u, 0u, 0u, 0u);
+        for (int u = 0; u < U; ++u)
+            s[u] = of_view(gv[u], blockIdx.y, runs.N) ? span[gv[u]] : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
         for (int u = 0; u < U; ++u)
             each_row(s[u], gv[u], more, xyzo, conic, alpha_min, cam, [&](int r, int c0, int c1) {
@@ -324,7 +325,6 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
             }
         }
     }
-    const uint32_t top = (uint32_t)runs.N * (uint32_t)vt.n - 1u;
     const int beg = runs.beg(blockIdx.y), cnt = runs.end(blockIdx.y) - beg;
     const uint32_t *sg = sorted_gv + (size_t)blockIdx.x * runs.N + beg;
     // bits of word i of row r's live tiles inside columns [c0, c1]
@@ -358,12 +358,12 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int i = pos + u * kBinThreads + tid;
-                gv[u] = i < cnt ? min(sg[i], top) : 0xffffffffu;
+                gv[u] = i < cnt ? sg[i] : 0xffffffffu;
             }
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 hit[u] = false;
-                if (gv[u] != 0xffffffffu) {
+                if (of_view(gv[u], blockIdx.x, runs.N)) {
                     const uint4 s = span[gv[u]];
                     const int n = (int)span_rows(s.x), x0 = (int)(s.x & 1023u), y0 = (int)((s.x >> 10) & 1023u);
                     if constexpr (CAPPED) {

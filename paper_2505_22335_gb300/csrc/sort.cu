@@ -346,8 +346,8 @@ cudaError_t radix_fixed(K **key_io, K **key_alt, uint32_t **val_io, uint32_t **v
 // ranks its items by ballots, publishes its 256 digit counts and finds the
 // items before it by walking back over the earlier tiles' published counts until
 // one holds its inclusive sum.  Every wait on a published count is bounded: a
-// wait that runs out sets *err and ends the CTA (its consumers clamp the ids
-// they read).  The first pass makes up the values (the positions) and the last
+// wait that runs out sets *err and ends the CTA (its consumers take no id on trust:
+// list_rules.cuh, k_gather_counts and k_emit).  The first pass makes up the values (the positions) and the last
 // one writes no keys.  Held by the ranking's ballots and the walk back, not by
 // its 16 bytes an item and pass: 8M keys 0.32 to 0.35 ms (0.38 with a histogram,
 // three scan kernels and a scatter a pass), 100k keys 47 us (130), where the 20
