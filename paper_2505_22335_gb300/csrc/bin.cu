@@ -223,19 +223,6 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *ws) {
     return before + incl - x;
 }
 
-// next free slot (and end) of every tile of the view in shared memory
-template <bool CAPPED> struct Slot;
-template <> struct Slot<true> {
-    uint32_t next, stop;
-    __device__ __forceinline__ bool room() const { return next < stop; }
-    __device__ __forceinline__ bool fits(uint32_t pos) const { return pos < stop; }
-};
-template <> struct Slot<false> {
-    uint32_t next;
-    __device__ __forceinline__ bool room() const { return true; }
-    __device__ __forceinline__ bool fits(uint32_t) const { return true; }
-};
-
 // shared bytes of k_bin_fill: queue, candidates, a slot and a mask word per
 // tile; capped: live bits and their summed-area table
 struct FillShape {
@@ -256,7 +243,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
                                                           const float4 *__restrict__ conic,
                                                           const uint32_t *__restrict__ prior,
                                                           const uint32_t *__restrict__ tot,
-                                                          const uint2 *__restrict__ ranges,
+                                                          const uint2 *__restrict__ ranges, uint32_t n,
                                                           uint32_t *__restrict__ lists, const int *__restrict__ gate) {
     if (gate && *gate == 0) return;
     extern __shared__ __align__(16) unsigned char sm[];
@@ -365,15 +352,15 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
                 hit[u] = false;
                 if (of_view(gv[u], blockIdx.x, runs.N)) {
                     const uint4 s = span[gv[u]];
-                    const int n = (int)span_rows(s.x), x0 = (int)(s.x & 1023u), y0 = (int)((s.x >> 10) & 1023u);
+                    const int nr = (int)span_rows(s.x), x0 = (int)(s.x & 1023u), y0 = (int)((s.x >> 10) & 1023u);
                     if constexpr (CAPPED) {
                         const uint32_t wide = s.x >> 25;
                         const int x1 = wide == kSpanWide ? tx : x0 + (int)wide + 1;
-                        const int y1 = n == (int)kSpanTall ? (int)(s.z >> 16) + 1 : y0 + n;
+                        const int y1 = nr == (int)kSpanTall ? (int)(s.z >> 16) + 1 : y0 + nr;
                         const int a = y0 * (tx + 1), b = y1 * (tx + 1);
-                        hit[u] = n && (int)sat[b + x1] - (int)sat[b + x0] - (int)sat[a + x1] + (int)sat[a + x0] > 0;
+                        hit[u] = nr && (int)sat[b + x1] - (int)sat[b + x0] - (int)sat[a + x1] + (int)sat[a + x0] > 0;
                     } else {
-                        hit[u] = n != 0;
+                        hit[u] = nr != 0;
                     }
                 }
                 hits[u] = __ballot_sync(0xffffffffu, hit[u]);
@@ -398,12 +385,12 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
         // the first 256 candidates' rows, numbered through
         const int m = min(nc, kBinThreads);
         const uint4 s4 = tid < m ? span[cand[tid]] : make_uint4(0u, 0u, 0u, 0u);
-        int n = (int)span_rows(s4.x);
-        if (n == (int)kSpanTall) n = (int)(s4.z >> 16) - (int)(s4.y >> 16) + 1;
-        const uint32_t first = block_scan((uint32_t)n, wsum);
+        int nr = (int)span_rows(s4.x);
+        if (nr == (int)kSpanTall) nr = (int)(s4.z >> 16) - (int)(s4.y >> 16) + 1;
+        const uint32_t first = block_scan((uint32_t)nr, wsum);
         s_first[tid] = (int)first;
         s_head[tid] = s4.x;
-        if (tid == kBinThreads - 1) s_first[kBinThreads] = (int)first + n;
+        if (tid == kBinThreads - 1) s_first[kBinThreads] = (int)first + nr;
         __syncthreads();
         const int rows = s_first[kBinThreads];
         for (int i0 = 0; i0 < rows;) {
@@ -457,7 +444,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
                     const uint32_t e = queue[j];
                     const Slot<CAPPED> sl = slot[e >> 8];
                     const uint32_t at = sl.next + __popc(mask[e >> 8] & ((1u << (e & 31u)) - 1u));
-                    if (sl.fits(at)) lists[at] = cand[e & 255u];
+                    if (sl.fits(at, n)) lists[at] = cand[e & 255u];
                 }
                 __syncthreads();
                 // the first Gaussian of each tile moves its slot on and clears its mask
@@ -561,7 +548,7 @@ cudaError_t bin_lists(const ViewTable &vt, float alpha_min, int N, const uint32_
     const cudaError_t e = allow_smem(kernel, capped ? fill_smem<true>(kMaxFill) : fill_smem<false>(kMaxFill));
     if (e != cudaSuccess) return e;
     kernel<<<dim3(vt.n, p.runs.nb), kBinThreads, smem, st>>>(vt, alpha_min, p.runs, sorted_gv, span, more, xyzo, conic,
-                                                       cnt, tot, ranges, lists, gate);
+                                                       cnt, tot, ranges, n, lists, gate);
     return cudaGetLastError();
 }
 

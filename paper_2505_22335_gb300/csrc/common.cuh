@@ -139,7 +139,8 @@ cudaError_t sorted_order_u64(uint64_t *key, uint64_t *key_alt, uint32_t *val, ui
 // t of trunc is set when it lost some.  Views of at most kMaxBinTiles tiles.
 // bin_count fills scratch (bin_scratch_bytes); bin_lists may follow it more
 // than once.  n: entries lists has room for (>= the tile instances if cap =
-// kNoListCap); gate: when non-null its kernels do nothing unless *gate != 0.
+// kNoListCap; 0: no instances); gate: when non-null its kernels do nothing unless
+// *gate != 0.
 constexpr int kMaxBinTiles = 8191;
 constexpr int kMaxListCap = 32767;
 constexpr uint32_t kNoListCap = 0xffffffffu;

@@ -26,8 +26,8 @@ cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *coun
                                  int total, cudaStream_t st);
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
                         const uint64_t *off, const uint2 *rect, const float4 *xyzo, const float4 *conic,
-                        uint32_t *ikey, uint32_t *ival, cudaStream_t st);
-cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaStream_t st);
+                        uint32_t *ikey, uint32_t *ival, uint32_t n_inst, cudaStream_t st);
+cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint32_t tiles, uint2 *ranges, cudaStream_t st);
 cudaError_t launch_clear_hits(const HitList &hits, size_t n_gv, float *g2, int n_feat, int num_sms, cudaStream_t st);
 cudaError_t launch_list_hits(const HitList &hits, size_t n_gv, cudaStream_t st);
 cudaError_t launch_project_bwd(const ViewTable &vt, const BlendParams &bp, int N, int n_sets, int direct, int n_feat,
@@ -155,6 +155,7 @@ struct ups_ctx {
     int *d_err = nullptr, *d_trunc_flag = nullptr;  // into d_words
     DevBuf trunc;                 // per-tile bit: the list cap cut the tile's list
     bool capped = false;          // the last forward capped its tile lists
+    bool rowwise = false;         // the last forward built its lists row by row (bin.cu)
     DevBuf lift_scr;              // feature-lifting scratch of one view
     DevBuf ssim_g;                // D-SSIM window-term maps of all colour planes
     DevBuf unc_scr;               // uncertainty-MLP patch scratch of all views
@@ -302,6 +303,8 @@ ups_status set_device(ups_ctx *c) {
     return UPS_OK;
 }
 
+constexpr size_t kListSpare = 1024;  // list entries beyond the counted instances
+
 // Tile lists of views too large for the row-wise kernels: every (tile,
 // Gaussian) instance of the depth-ordered Gaussian-views dv is written, then
 // sorted by tile (stable: depth order is kept inside each tile).
@@ -321,7 +324,7 @@ ups_status instance_lists(ups_ctx *c, const uint32_t *dv, size_t total, cudaStre
     uint32_t *iv = c->ival0.as<uint32_t>(), *iv_alt = c->ival1.as<uint32_t>();
     stage_begin(c, "emit", st);
     UPS_CUDA(c, launch_emit(vt, c->bp, c->N, (int)total, dv, c->off.as<uint64_t>(), c->rect.as<uint2>(),
-                            c->xyzo.as<float4>(), c->conic.as<float4>(), ik, iv, st));
+                            c->xyzo.as<float4>(), c->conic.as<float4>(), ik, iv, (uint32_t)n_inst, st));
     stage_end(c, st, 1);
     stage_begin(c, "tile_sort", st);
     UPS_CUDA(c, radix_sort_u32(&ik, &ik_alt, &iv, &iv_alt, n_inst, c->key_bits, c->sort, st));
@@ -330,7 +333,7 @@ ups_status instance_lists(ups_ctx *c, const uint32_t *dv, size_t total, cudaStre
     c->ival_sorted = iv;
     stage_begin(c, "ranges", st);
     UPS_CUDA(c, cudaMemsetAsync(c->ranges.ptr, 0, (size_t)vt.total_tiles * sizeof(uint2), st));
-    UPS_CUDA(c, launch_ranges(ik, (uint32_t)n_inst, c->ranges.as<uint2>(), st));
+    UPS_CUDA(c, launch_ranges(ik, (uint32_t)n_inst, (uint32_t)vt.total_tiles, c->ranges.as<uint2>(), st));
     stage_end(c, st, n_inst ? 1 : 0);
     return UPS_OK;
 }
@@ -364,12 +367,12 @@ ups_status loss_views(ups_ctx *c, const ups_images *img, const ups_targets *tgt,
     return UPS_OK;
 }
 // Entries in the tile lists of the last forward (a capped forward keeps
-// fewer than it emitted unless the GPU rebuilt them whole: *refilled).
+// fewer than there are instances unless the GPU rebuilt them whole: *refilled).
 // Synchronises the ctx stream.
 ups_status listed_entries(ups_ctx *c, size_t *listed, int *refilled) {
     *listed = c->n_inst;
     *refilled = 0;
-    if (!c->capped) return UPS_OK;
+    if (!c->rowwise) return UPS_OK;
     UPS_CUDA(c, cudaSetDevice(c->device));
     UPS_CUDA(c, cudaStreamSynchronize(c->last_stream));
     uint2 last;
@@ -378,7 +381,7 @@ ups_status listed_entries(ups_ctx *c, size_t *listed, int *refilled) {
                            cudaMemcpyDeviceToHost));
     UPS_CUDA(c, cudaMemcpy(&flag, c->d_trunc_flag, sizeof(int), cudaMemcpyDeviceToHost));
     *listed = last.y;
-    *refilled = flag != 0;
+    *refilled = c->capped && flag != 0;
     return UPS_OK;
 }
 
@@ -598,7 +601,7 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     UPS_CUDA(c, c->ranges.reserve((size_t)vt.total_tiles * sizeof(uint2)));
     // tile lists straight from the depth order, unless a view has more tiles
     // than the row-wise kernels take
-    const bool rowwise = bin_supported(vt);
+    const bool rowwise = c->rowwise = bin_supported(vt);
     if (rowwise) {
         UPS_CUDA(c, c->span.reserve(total * sizeof(uint4)));
         UPS_CUDA(c, c->more.reserve(total * kSpanMore * sizeof(uint4)));
@@ -655,13 +658,17 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
                              : (uint32_t)(c->cfg.list_cap == 0 ? 1024 : c->cfg.list_cap);
     c->ikey_sorted = nullptr;  // rebuilt from the ranges when inspected
     auto lists = [&](uint32_t keep, const int *gate) {
+        const size_t room = n_inst ? std::min<size_t>(c->lists.bytes / sizeof(uint32_t), UINT32_MAX) : 0;
         return bin_lists(vt, c->bp.alpha_min, c->N, dv, span, more, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                         c->bin_scr.ptr, keep, (uint32_t)n_inst, c->ranges.as<uint2>(), c->trunc.as<uint32_t>(),
+                         c->bin_scr.ptr, keep, (uint32_t)room, c->ranges.as<uint2>(), c->trunc.as<uint32_t>(),
                          c->lists.as<uint32_t>(), c->num_sms, st, gate);
     };
     if (rowwise) {
-        // room for every instance: a capped list may have to be rebuilt whole
-        UPS_CUDA(c, c->lists.reserve(std::max<size_t>(n_inst, 1) * sizeof(uint32_t)));
+        // room for every instance: a capped list may have to be rebuilt whole.  The
+        // projection counted them; the list kernels evaluate the rows of the tallest and
+        // widest Gaussians again, where a tile that the margin decides may come out another
+        // way, so a few more find room.
+        UPS_CUDA(c, c->lists.reserve(((size_t)n_inst + kListSpare) * sizeof(uint32_t)));
         stage_begin(c, "tile_lists", st);
         UPS_CUDA(c, lists(cap, nullptr));
         stage_end(c, st, n_inst ? 2 : 1);

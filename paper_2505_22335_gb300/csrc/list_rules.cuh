@@ -19,4 +19,21 @@ namespace ups {
 // that view's columns and rows, and its Gaussian set past the end.
 UPS_HD bool of_view(uint32_t gv, uint32_t v, uint32_t N) { return gv - v * N < N; }
 
+// Next free position (and end) of a tile's list while a run of Gaussians is filled in; n:
+// entries that the list buffer has room for.  An uncapped list has no end of its own: its
+// positions come from counts that are taken again from an order that may repeat an id,
+// or (for Gaussians whose rows are evaluated again) by another kernel than the one that
+// sized the buffer, so every position is held against the buffer.
+template <bool CAPPED> struct Slot;
+template <> struct Slot<true> {
+    uint32_t next, stop;  // stop <= n
+    UPS_HD bool room() const { return next < stop; }
+    UPS_HD bool fits(uint32_t pos, uint32_t) const { return pos < stop; }
+};
+template <> struct Slot<false> {
+    uint32_t next;
+    UPS_HD bool room() const { return true; }
+    UPS_HD bool fits(uint32_t pos, uint32_t n) const { return pos < n; }
+};
+
 }  // namespace ups

@@ -40,8 +40,8 @@ cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *coun
                                  int total, cudaStream_t st);
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
                         const uint64_t *off, const uint2 *rect, const float4 *xyzo, const float4 *conic,
-                        uint32_t *ikey, uint32_t *ival, cudaStream_t st);
-cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaStream_t st);
+                        uint32_t *ikey, uint32_t *ival, uint32_t n_inst, cudaStream_t st);
+cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint32_t tiles, uint2 *ranges, cudaStream_t st);
 cudaError_t launch_composite_fwd(const ViewTable &vt, const BlendParams &bp, int n_feat, int N,
                                  int per_view, const uint2 *ranges, const uint32_t *ival,
                                  const float4 *xyzo, const float4 *conic, const float4 *color,
@@ -219,11 +219,11 @@ extern "C" ups_status ups_render_forward_static(const ups_config *cfg, const ups
     NA_CUDA(cudaStreamSynchronize(st));
     if (n_inst > kMaxInst)
         return fail(UPS_ERR_CAPACITY, std::to_string(n_inst) + " tile instances exceed 524288");
-    NA_CUDA(launch_emit(vt, bp, N, (int)total, dv, off, rect, xyzo, conic, ik, iv, st));
+    NA_CUDA(launch_emit(vt, bp, N, (int)total, dv, off, rect, xyzo, conic, ik, iv, (uint32_t)n_inst, st));
     NA_CUDA(radix_sort_u32_fixed(&ik, &ik_alt, &iv, &iv_alt, (size_t)n_inst,
                                  bits_for((size_t)vt.total_tiles), sort_scr, kSortScratch, st));
     NA_CUDA(cudaMemsetAsync(ranges, 0, (size_t)vt.total_tiles * sizeof(uint2), st));
-    NA_CUDA(launch_ranges(ik, (uint32_t)n_inst, ranges, st));
+    NA_CUDA(launch_ranges(ik, (uint32_t)n_inst, (uint32_t)vt.total_tiles, ranges, st));
     NA_CUDA(launch_composite_fwd(vt, bp, nf, N, per_view, ranges, iv, xyzo, conic,
                                  reinterpret_cast<const float4 *>(g->color), g->feat, *out, 0, st));
     return UPS_OK;

@@ -274,7 +274,9 @@ __global__ void k_gather_counts(const uint32_t *__restrict__ sorted_gv,
 // so stores are coalesced whatever the per-Gaussian tile counts are.  Each
 // owner lane first tabulates its Gaussian's met columns per tile row (first
 // column and running instance count) in shared memory, up to kEmitRows rows;
-// taller Gaussians (rare) recompute the rows per instance.
+// taller Gaussians (rare) recompute the rows per instance.  The buffers hold the
+// n_inst instances that the projection counted; an order that a lost wait left with
+// repeated ids adds up to more or fewer.
 constexpr int kEmitRows = 8;
 
 __global__ void __launch_bounds__(256) k_emit(ViewTable vt, BlendParams bp, int N, int total,
@@ -284,7 +286,7 @@ __global__ void __launch_bounds__(256) k_emit(ViewTable vt, BlendParams bp, int 
                                               const float4 *__restrict__ xyzo,
                                               const float4 *__restrict__ conic,
                                               uint32_t *__restrict__ ikey,
-                                              uint32_t *__restrict__ ival) {
+                                              uint32_t *__restrict__ ival, uint32_t n_inst) {
     __shared__ uint32_t s_rows[256 / 32][32][kEmitRows];  // first column | (instances before the row << 16)
     const unsigned full = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(256) k_emit(ViewTable vt, BlendParams bp, int 
         const uint32_t r0 = __shfl_sync(full, rc.x, L);
         const uint32_t r1 = __shfl_sync(full, rc.y, L);
         const uint64_t oL = __shfl_sync(full, o, L);
-        if (i < o_end) {
+        if (i < o_end && i < n_inst) {
             const int v = (int)(g / (uint32_t)N);
             const DevView &cam = vt.v[v];
             const int x0 = r0 & 0xffff, y0 = r0 >> 16, x1 = r1 & 0xffff, y1 = r1 >> 16;
@@ -361,12 +363,19 @@ __global__ void __launch_bounds__(256) k_emit(ViewTable vt, BlendParams bp, int 
             ival[i] = g;
         }
     }
+    // fewer instances than the buffers were sized for: no tile's
+    if (s0 + 32 >= total)
+        for (uint64_t i = o_end + lane; i < n_inst; i += 32) {
+            ikey[i] = 0xffffffffu;
+            ival[i] = 0u;
+        }
 }
 
-__global__ void k_ranges(const uint32_t *__restrict__ ikey, uint32_t n, uint2 *__restrict__ ranges) {
+__global__ void k_ranges(const uint32_t *__restrict__ ikey, uint32_t n, uint32_t tiles, uint2 *__restrict__ ranges) {
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     uint32_t k = ikey[i];
+    if (k >= tiles) return;
     if (i == 0 || ikey[i - 1] != k) ranges[k].x = i;
     if (i == n - 1 || ikey[i + 1] != k) ranges[k].y = i + 1;
 }
@@ -682,15 +691,15 @@ cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *coun
 
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
                         const uint64_t *off, const uint2 *rect, const float4 *xyzo, const float4 *conic,
-                        uint32_t *ikey, uint32_t *ival, cudaStream_t st) {
+                        uint32_t *ikey, uint32_t *ival, uint32_t n_inst, cudaStream_t st) {
     if (total == 0) return cudaSuccess;
-    k_emit<<<(total + 255) / 256, 256, 0, st>>>(vt, bp, N, total, sorted_gv, off, rect, xyzo, conic, ikey, ival);
+    k_emit<<<(total + 255) / 256, 256, 0, st>>>(vt, bp, N, total, sorted_gv, off, rect, xyzo, conic, ikey, ival, n_inst);
     return cudaGetLastError();
 }
 
-cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint2 *ranges, cudaStream_t st) {
+cudaError_t launch_ranges(const uint32_t *ikey, uint32_t n, uint32_t tiles, uint2 *ranges, cudaStream_t st) {
     if (n == 0) return cudaSuccess;
-    k_ranges<<<(n + 255) / 256, 256, 0, st>>>(ikey, n, ranges);
+    k_ranges<<<(n + 255) / 256, 256, 0, st>>>(ikey, n, tiles, ranges);
     return cudaGetLastError();
 }
 

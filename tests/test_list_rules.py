@@ -62,3 +62,79 @@ int main() {
     return 0;
 }
 """)
+
+
+def test_list_positions_stay_in_the_buffer(tmp_path):
+    # The arithmetic of bin.cu (counts a run, their prefix, ranges, fill) over orders that
+    # repeat ids: every position that the rules let through lies in the buffer, and of a
+    # sound order every entry is kept.
+    run(tmp_path, """
+template <bool CAPPED> int fill(const std::vector<uint32_t> &order, const std::vector<std::vector<int>> &tiles_of,
+                                int tiles, uint32_t cap, uint32_t n, bool sound) {
+    const int N = (int)order.size(), R = 64, nb = (N + R - 1) / R;
+    std::vector<uint32_t> cnt((size_t)nb * tiles), tot(tiles), list(n, ~0u);
+    for (int i = 0; i < N; ++i)
+        if (of_view(order[i], 0, N))
+            for (int t : tiles_of[order[i]]) cnt[(size_t)(i / R) * tiles + t]++;
+    for (int t = 0; t < tiles; ++t)
+        for (int b = 0; b < nb; ++b) {
+            const uint32_t c = cnt[(size_t)b * tiles + t];
+            cnt[(size_t)b * tiles + t] = tot[t];
+            tot[t] += c;
+        }
+    std::vector<std::pair<uint32_t, uint32_t>> rg(tiles);
+    uint32_t at = 0, kept = 0;
+    for (int t = 0; t < tiles; ++t) {
+        const uint32_t k = std::min(tot[t], cap);
+        rg[t] = {std::min(at, n), std::min(at + k, n)};
+        at += k;
+    }
+    for (int b = 0; b < nb; ++b) {
+        std::vector<Slot<CAPPED>> slot(tiles);
+        for (int t = 0; t < tiles; ++t) {
+            slot[t].next = rg[t].first + std::min(cnt[(size_t)b * tiles + t], rg[t].second - rg[t].first);
+            if constexpr (CAPPED) slot[t].stop = rg[t].second;
+        }
+        for (int i = b * R; i < std::min(N, (b + 1) * R); ++i) {
+            if (!of_view(order[i], 0, N)) continue;
+            for (int t : tiles_of[order[i]]) {
+                const uint32_t pos = slot[t].next++;
+                if (!slot[t].fits(pos, n)) continue;
+                CHECK(pos < list.size());
+                list[pos] = order[i];
+                ++kept;
+            }
+        }
+    }
+    if (sound) CHECK(kept == std::min(at, n));
+    return 0;
+}
+
+int main() {
+    std::mt19937 rng(2);
+    for (int trial = 0; trial < 60; ++trial) {
+        const int N = 1 + rng() % 700, tiles = 1 + rng() % 40;
+        std::vector<std::vector<int>> tiles_of(N);
+        uint32_t n = 0;
+        for (auto &t : tiles_of) {
+            for (int k = rng() % 4; k > 0; --k) t.push_back(rng() % tiles);
+            n += (uint32_t)t.size();
+        }
+        std::vector<uint32_t> order(N);
+        for (int i = 0; i < N; ++i) order[i] = i;
+        std::shuffle(order.begin(), order.end(), rng);
+        uint32_t most = 0;  // the id with the most tiles: repeated, more entries than the buffer has
+        for (int i = 0; i < N; ++i)
+            if (tiles_of[i].size() > tiles_of[most].size()) most = i;
+        for (int broken = 0; broken < 2; ++broken) {
+            if (broken)
+                for (int i = 0; i < N; ++i)
+                    if (rng() % 3 == 0) order[i] = rng() % 4 ? most : rng();
+            if (fill<false>(order, tiles_of, tiles, ~0u, n, !broken)) return 1;
+            for (uint32_t cap : {1u, 7u, 1000u})
+                if (fill<true>(order, tiles_of, tiles, cap, n, !broken)) return 1;
+        }
+    }
+    return 0;
+}
+""")
