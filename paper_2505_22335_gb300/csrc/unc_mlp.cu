@@ -166,7 +166,8 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
         // Pass 2 steps the pre-activation along x, which rounds it another way than the
         // corner-by-corner sum of pass 1 (both within 14 roundings of the magnitudes
         // summed, 2^-20 of their sum): where a unit is nearer to 0 than that, pass 2
-        // takes pass 1's sum, so that both take the same units for on.
+        // takes pass 1's sum, so that both take the same units for on (also where the
+        // steps are not numbers: corner values that are infinite).
         float near0 = 0.f;
         {
             const float4 b = reinterpret_cast<const float4 *>(s_b1)[lane];
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                         float u0, u1, u2, u3;
                         f2_split(za, u0, u1);
                         f2_split(zb, u2, u3);
-                        if (fminf(fminf(fabsf(u0), fabsf(u1)), fminf(fabsf(u2), fabsf(u3))) <= near0) {
+                        if (!(fminf(fminf(fabsf(u0), fabsf(u1)), fminf(fabsf(u2), fabsf(u3))) > near0)) {
                             const float wt[4] = {(1.f - t.y) * (1.f - ay), t.y * (1.f - ay), (1.f - t.y) * ay, t.y * ay};
                             za = bb01;
                             zb = bb23;
@@ -283,8 +284,9 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                         S0b = f2_add(S0b, mb);
                         S1a = f2_fma(ma, ax2, S1a);
                         S1b = f2_fma(mb, ax2, S1b);
-                        a_dw01 = f2_fma(ma, za, a_dw01);
-                        a_dw23 = f2_fma(mb, zb, a_dw23);
+                        // the hidden values, not z: an off unit's z may be infinite or NaN
+                        a_dw01 = f2_fma(ma, f2_make(fmaxf(u0, 0.f), fmaxf(u1, 0.f)), a_dw01);
+                        a_dw23 = f2_fma(mb, f2_make(fmaxf(u2, 0.f), fmaxf(u3, 0.f)), a_dw23);
                     }
                     const f2 neg = f2_make(-1.f, -1.f);
                     const f2 La = f2_fma(neg, S1a, S0a), Lb = f2_fma(neg, S1b, S0b);
