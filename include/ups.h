@@ -76,7 +76,7 @@ typedef struct {
                          pixel is still open at the end of a cut list: the forward
                          then sorts that batch again without the cap and blends it
                          again (ups_stats.list_refills).  Batches with a view of
-                         more than 8191 tiles are never capped. */
+                         more than 16384 tiles are never capped. */
     int opacity_tanh; /* 1: decoded opacity o = tanh(y) (the Scaffold-GS decode the
                          paper cites for Eq. 8-9) instead of sigmoid(y); the
                          projection's cull of o < alpha_min then drops every

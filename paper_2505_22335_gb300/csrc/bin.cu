@@ -226,7 +226,7 @@ __device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t *ws) {
 // shared bytes of k_bin_fill: queue, candidates, a slot and a mask word per
 // tile; capped: live bits and their summed-area table
 struct FillShape {
-    int tiles, live_words, sat;  // largest of the views
+    int tiles, live_words, sat;  // largest of the views (of their bands)
 };
 template <bool CAPPED>
 size_t fill_smem(const FillShape &f) {
@@ -234,7 +234,9 @@ size_t fill_smem(const FillShape &f) {
            (CAPPED ? (size_t)f.live_words * 4 + (size_t)f.sat * 2 : 0);
 }
 
-template <bool CAPPED>
+// BANDS: grid.x is views x bands; a CTA fills the tiles of one band of its view's rows,
+// ceil(tiles_y / bands) rows each (the last ones may have none).  See plan_of.
+template <bool CAPPED, bool BANDS>
 __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float alpha_min, Runs runs,
                                                           const uint32_t *__restrict__ sorted_gv,
                                                           const uint4 *__restrict__ span,
@@ -244,7 +246,8 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
                                                           const uint32_t *__restrict__ prior,
                                                           const uint32_t *__restrict__ tot,
                                                           const uint2 *__restrict__ ranges, uint32_t n,
-                                                          uint32_t *__restrict__ lists, const int *__restrict__ gate) {
+                                                          uint32_t *__restrict__ lists, const int *__restrict__ gate,
+                                                          int bands) {
     if (gate && *gate == 0) return;
     extern __shared__ __align__(16) unsigned char sm[];
     __shared__ uint32_t wsum[2 * kBinWarps];
@@ -254,8 +257,14 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
     __shared__ int s_first_window;
     // runs along grid.y: the nearest runs of every view, which hold most of the
     // entries, start first
-    const DevView &cam = vt.v[blockIdx.x];
-    const int tx = cam.tiles_x, ty = cam.tiles_y, tiles = tx * ty;
+    const int view = BANDS ? blockIdx.x / bands : blockIdx.x;
+    const DevView &cam = vt.v[view];
+    // rows and tiles of the band, counted from its first row b0 and first tile t0
+    const int per_band = BANDS ? (cam.tiles_y + bands - 1) / bands : cam.tiles_y;
+    const int b0 = BANDS ? ((int)blockIdx.x - view * bands) * per_band : 0;
+    const int tx = cam.tiles_x, ty = BANDS ? min(per_band, cam.tiles_y - b0) : cam.tiles_y, tiles = tx * ty;
+    const int t0 = cam.tile_base + b0 * tx;
+    if (BANDS && ty <= 0) return;
     const int lw = (tx + 31) >> 5;  // words of a row's live bits
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const uint32_t lt_mask = (1u << lane) - 1u;
@@ -267,15 +276,16 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
     uint16_t *sat = reinterpret_cast<uint16_t *>(live + lw * ty);  // capped: [ty + 1][tx + 1] live tiles above and left
     // the tiles' slots before this run; leave if none takes anything from it
     {
-        const uint32_t *pr = prior + (size_t)runs.nb * cam.tile_base + (size_t)blockIdx.y * tiles;
-        const uint32_t *pn = (int)blockIdx.y == runs.nb - 1 ? tot + cam.tile_base : pr + tiles;
+        const int all = tx * cam.tiles_y;  // of the view
+        const uint32_t *pr = prior + (size_t)runs.nb * cam.tile_base + (size_t)blockIdx.y * all + b0 * tx;
+        const uint32_t *pn = (int)blockIdx.y == runs.nb - 1 ? tot + t0 : pr + all;
         bool any = false;
         if constexpr (CAPPED) {
             for (int i = tid; i < lw * ty; i += kBinThreads) live[i] = 0u;
             __syncthreads();
         }
         for (int t = tid; t < tiles; t += kBinThreads) {
-            const uint2 r = ranges[cam.tile_base + t];
+            const uint2 r = ranges[t0 + t];
             const uint32_t p = pr[t];
             const uint32_t at = r.x + min(p, r.y - r.x);
             const bool takes = pn[t] > p && at < r.y;
@@ -313,7 +323,7 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
         }
     }
     const int beg = runs.beg(blockIdx.y), cnt = runs.end(blockIdx.y) - beg;
-    const uint32_t *sg = sorted_gv + (size_t)blockIdx.x * runs.N + beg;
+    const uint32_t *sg = sorted_gv + (size_t)view * runs.N + beg;
     // bits of word i of row r's live tiles inside columns [c0, c1]
     auto live_word = [&](const RowItem &t, int i) {
         uint32_t b = live[t.r * lw + i];
@@ -350,17 +360,19 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 hit[u] = false;
-                if (of_view(gv[u], blockIdx.x, runs.N)) {
+                if (of_view(gv[u], view, runs.N)) {
                     const uint4 s = span[gv[u]];
                     const int nr = (int)span_rows(s.x), x0 = (int)(s.x & 1023u), y0 = (int)((s.x >> 10) & 1023u);
+                    // rows [ya, yb) of the band
+                    const int y1 = nr == (int)kSpanTall ? (int)(s.z >> 16) + 1 : y0 + nr;
+                    const int ya = BANDS ? max(y0 - b0, 0) : y0, yb = BANDS ? min(y1 - b0, ty) : y1;
+                    hit[u] = nr && (!BANDS || ya < yb);
                     if constexpr (CAPPED) {
                         const uint32_t wide = s.x >> 25;
                         const int x1 = wide == kSpanWide ? tx : x0 + (int)wide + 1;
-                        const int y1 = nr == (int)kSpanTall ? (int)(s.z >> 16) + 1 : y0 + nr;
-                        const int a = y0 * (tx + 1), b = y1 * (tx + 1);
-                        hit[u] = nr && (int)sat[b + x1] - (int)sat[b + x0] - (int)sat[a + x1] + (int)sat[a + x0] > 0;
-                    } else {
-                        hit[u] = nr != 0;
+                        const int a = ya * (tx + 1), b = yb * (tx + 1);
+                        hit[u] = hit[u] &&
+                                 (int)sat[b + x1] - (int)sat[b + x0] - (int)sat[a + x1] + (int)sat[a + x0] > 0;
                     }
                 }
                 hits[u] = __ballot_sync(0xffffffffu, hit[u]);
@@ -382,11 +394,15 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
         }
         __syncthreads();
         if (nc == 0) break;
-        // the first 256 candidates' rows, numbered through
+        // the first 256 candidates' rows (in the band: one at least), numbered through
         const int m = min(nc, kBinThreads);
         const uint4 s4 = tid < m ? span[cand[tid]] : make_uint4(0u, 0u, 0u, 0u);
         int nr = (int)span_rows(s4.x);
         if (nr == (int)kSpanTall) nr = (int)(s4.z >> 16) - (int)(s4.y >> 16) + 1;
+        if (BANDS && tid < m) {
+            const int y0 = (int)((s4.x >> 10) & 1023u);
+            nr = min(y0 + nr, b0 + ty) - max(y0, b0);
+        }
         const uint32_t first = block_scan((uint32_t)nr, wsum);
         s_first[tid] = (int)first;
         s_head[tid] = s4.x;
@@ -402,8 +418,12 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
             for (int step = kBinThreads / 2; step >= 1; step >>= 1)
                 if (s_first[L + step] <= i) L += step;
             RowItem t{0, 1, 0};
-            if (in)
-                t = row_item(cand[L], s_head[L], i - s_first[L], span, more, xyzo, conic, alpha_min, cam);
+            if (in) {
+                const uint32_t head = s_head[L];
+                const int skip = BANDS ? max(b0 - (int)((head >> 10) & 1023u), 0) : 0;  // rows above the band
+                t = row_item(cand[L], head, i - s_first[L] + skip, span, more, xyzo, conic, alpha_min, cam);
+                t.r -= b0;
+            }
             const uint32_t c = t.c0 <= t.c1 ? entries(t) : 0u;
             uint32_t o = block_scan(c, wsum);
             // rows whose entries fit the queue (all but the last few of a step, if any are left)
@@ -476,9 +496,20 @@ __global__ void __launch_bounds__(kBinThreads) k_bin_fill(ViewTable vt, float al
 
 struct Plan {
     Runs runs;
+    int bands, most_tiles;  // of the fill; tiles of the largest view
     FillShape fill;
     size_t count_smem;
 };
+
+// A view of more than kBandless tiles is filled in bands of about kBandTiles: the state
+// of its tiles (14 bytes each) would take most of an SM's shared memory, or more than
+// there is, and leave it one CTA.  One view of 2560x1440 (14,400 tiles): 300k Gaussians
+// (13.8M instances) lists 0.27 ms and 1.12 the frame, where one band with the ends of the
+// lists read from global memory took 0.59 and writing and bucket sorting every instance
+// 1.11 (2.10); 1M small faint ones (4.8M instances) 0.33 against 0.67 and 0.41.
+constexpr int kBandless = 8191, kBandTiles = 4096;
+// tile sides are at most this (16,384 pixels)
+constexpr int kMaxSide = 1024;
 
 // Runs of 512 for the nearest eighth of a view and 4096 behind it; a batch with
 // fewer than four runs of 2048 an SM takes short ones throughout, down to 128
@@ -494,21 +525,35 @@ Plan plan_of(const ViewTable &vt, int N, int num_sms) {
     while (N / r.r2 > 30000) r.r1 <<= 1, r.r2 <<= 1;  // runs lie along grid.y
     r.nb1 = r.r1 == r.r2 ? 0 : N / 8 / r.r1;
     r.nb = r.nb1 + (N - r.nb1 * r.r1 + r.r2 - 1) / r.r2;
+    for (int v = 0; v < vt.n; ++v) p.most_tiles = std::max(p.most_tiles, vt.v[v].tiles_x * vt.v[v].tiles_y);
+    p.bands = p.most_tiles <= kBandless ? 1 : (p.most_tiles + kBandTiles - 1) / kBandTiles;
     for (int v = 0; v < vt.n; ++v) {
         const DevView &c = vt.v[v];
-        p.fill.tiles = std::max(p.fill.tiles, c.tiles_x * c.tiles_y);
-        p.fill.live_words = std::max(p.fill.live_words, (c.tiles_x + 31) / 32 * c.tiles_y);
-        p.fill.sat = std::max(p.fill.sat, (c.tiles_x + 1) * (c.tiles_y + 1));
+        const int rows = (c.tiles_y + p.bands - 1) / p.bands;
+        p.fill.tiles = std::max(p.fill.tiles, c.tiles_x * rows);
+        p.fill.live_words = std::max(p.fill.live_words, (c.tiles_x + 31) / 32 * rows);
+        p.fill.sat = std::max(p.fill.sat, (c.tiles_x + 1) * (rows + 1));
         p.count_smem = std::max(p.count_smem, (size_t)(c.tiles_x + 1) * c.tiles_y * sizeof(int));
     }
     return p;
 }
 
-// The largest shared memory of a view: kMaxBinTiles tiles, at most kMaxSide a side
-// (16,384 pixels).
-constexpr int kMaxSide = 1024;
-constexpr FillShape kMaxFill{kMaxBinTiles, kMaxBinTiles / 32 + kMaxSide, kMaxBinTiles + 2 * kMaxSide + 1};
+// The largest shape of a view or band (a band's last row may pass kBandTiles, but not
+// kBandless), at most kMaxSide tiles a side.
+constexpr FillShape kMaxFill{kBandless, kBandless / 32 + kMaxSide, kBandless + 2 * kMaxSide + 1};
 constexpr size_t kMaxCountSmem = (size_t)(kMaxBinTiles + kMaxSide) * sizeof(int);
+
+template <bool CAPPED, bool BANDS>
+cudaError_t launch_fill(const ViewTable &vt, float alpha_min, const Plan &p, const uint32_t *sorted_gv,
+                        const uint4 *span, const uint4 *more, const float4 *xyzo, const float4 *conic,
+                        const uint32_t *cnt, const uint32_t *tot, const uint2 *ranges, uint32_t n, uint32_t *lists,
+                        const int *gate, cudaStream_t st) {
+    const cudaError_t e = allow_smem(k_bin_fill<CAPPED, BANDS>, fill_smem<CAPPED>(kMaxFill));
+    if (e != cudaSuccess) return e;
+    k_bin_fill<CAPPED, BANDS><<<dim3(vt.n * p.bands, p.runs.nb), kBinThreads, fill_smem<CAPPED>(p.fill), st>>>(
+        vt, alpha_min, p.runs, sorted_gv, span, more, xyzo, conic, cnt, tot, ranges, n, lists, gate, p.bands);
+    return cudaGetLastError();
+}
 
 }  // namespace
 
@@ -531,7 +576,7 @@ cudaError_t bin_count(const ViewTable &vt, float alpha_min, int N, const uint32_
     if (e != cudaSuccess) return e;
     k_bin_count<<<dim3(p.runs.nb, vt.n), kBinThreads, p.count_smem, st>>>(vt, alpha_min, p.runs, sorted_gv, span,
                                                                      more, xyzo, conic, cnt);
-    k_bin_prefix<<<dim3((p.fill.tiles + 31) / 32, vt.n), 32 * kPrefWarps, 0, st>>>(vt, p.runs.nb, cnt, tot);
+    k_bin_prefix<<<dim3((p.most_tiles + 31) / 32, vt.n), 32 * kPrefWarps, 0, st>>>(vt, p.runs.nb, cnt, tot);
     return cudaGetLastError();
 }
 
@@ -542,14 +587,9 @@ cudaError_t bin_lists(const ViewTable &vt, float alpha_min, int N, const uint32_
     uint32_t *tot = static_cast<uint32_t *>(scratch), *cnt = tot + vt.total_tiles;
     k_bin_ranges<<<1, kRangeThreads, 0, st>>>(tot, vt.total_tiles, cap, n, ranges, trunc, gate);
     if (n == 0) return cudaGetLastError();
-    const bool capped = cap != kNoListCap;
-    const size_t smem = capped ? fill_smem<true>(p.fill) : fill_smem<false>(p.fill);
-    const auto kernel = capped ? k_bin_fill<true> : k_bin_fill<false>;
-    const cudaError_t e = allow_smem(kernel, capped ? fill_smem<true>(kMaxFill) : fill_smem<false>(kMaxFill));
-    if (e != cudaSuccess) return e;
-    kernel<<<dim3(vt.n, p.runs.nb), kBinThreads, smem, st>>>(vt, alpha_min, p.runs, sorted_gv, span, more, xyzo, conic,
-                                                       cnt, tot, ranges, n, lists, gate);
-    return cudaGetLastError();
+    const auto fill = cap == kNoListCap ? (p.bands > 1 ? launch_fill<false, true> : launch_fill<false, false>)
+                                        : (p.bands > 1 ? launch_fill<true, true> : launch_fill<true, false>);
+    return fill(vt, alpha_min, p, sorted_gv, span, more, xyzo, conic, cnt, tot, ranges, n, lists, gate, st);
 }
 
 namespace {

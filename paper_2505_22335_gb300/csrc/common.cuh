@@ -141,7 +141,7 @@ cudaError_t sorted_order_u64(uint64_t *key, uint64_t *key_alt, uint32_t *val, ui
 // than once.  n: entries lists has room for (>= the tile instances if cap =
 // kNoListCap; 0: no instances); gate: when non-null its kernels do nothing unless
 // *gate != 0.
-constexpr int kMaxBinTiles = 8191;
+constexpr int kMaxBinTiles = 16384;
 constexpr int kMaxListCap = 32767;
 constexpr uint32_t kNoListCap = 0xffffffffu;
 bool bin_supported(const ViewTable &vt);
