@@ -166,8 +166,9 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
         // Pass 2 steps the pre-activation along x, which rounds it another way than the
         // corner-by-corner sum of pass 1 (both within 14 roundings of the magnitudes
         // summed, 2^-20 of their sum): where a unit is nearer to 0 than that, pass 2
-        // takes pass 1's sum, so that both take the same units for on (also where the
-        // steps are not numbers: corner values that are infinite).
+        // takes pass 1's sum, so that both take the same units for on.  Values that are not
+        // finite always take it, and there the hidden values and not z go into dL/dw2: zero
+        // times an off unit's z would not be zero.
         float near0 = 0.f;
         {
             const float4 b = reinterpret_cast<const float4 *>(s_b1)[lane];
@@ -181,6 +182,7 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                 m[3] += fabsf(z.w);
             }
             near0 = fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3])) * 9.5367431640625e-7f;
+            if (!((m[0] + m[1]) + (m[2] + m[3]) < INFINITY)) near0 = INFINITY;
         }
         f2 aD[4][2] = {};
         // units of at most kUnit pixels: bw columns, br rows
@@ -277,6 +279,8 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                             }
                             f2_split(za, u0, u1);
                             f2_split(zb, u2, u3);
+                            za = f2_make(fmaxf(u0, 0.f), fmaxf(u1, 0.f));
+                            zb = f2_make(fmaxf(u2, 0.f), fmaxf(u3, 0.f));
                         }
                         const f2 ma = f2_make(u0 > 0.f ? t.x : 0.f, u1 > 0.f ? t.x : 0.f);
                         const f2 mb = f2_make(u2 > 0.f ? t.x : 0.f, u3 > 0.f ? t.x : 0.f);
@@ -284,9 +288,8 @@ __global__ void __launch_bounds__(32 * kUWarps, 4) k_unc_cells(
                         S0b = f2_add(S0b, mb);
                         S1a = f2_fma(ma, ax2, S1a);
                         S1b = f2_fma(mb, ax2, S1b);
-                        // the hidden values, not z: an off unit's z may be infinite or NaN
-                        a_dw01 = f2_fma(ma, f2_make(fmaxf(u0, 0.f), fmaxf(u1, 0.f)), a_dw01);
-                        a_dw23 = f2_fma(mb, f2_make(fmaxf(u2, 0.f), fmaxf(u3, 0.f)), a_dw23);
+                        a_dw01 = f2_fma(ma, za, a_dw01);
+                        a_dw23 = f2_fma(mb, zb, a_dw23);
                     }
                     const f2 neg = f2_make(-1.f, -1.f);
                     const f2 La = f2_fma(neg, S1a, S0a), Lb = f2_fma(neg, S1b, S0b);

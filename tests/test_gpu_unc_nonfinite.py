@@ -2,7 +2,7 @@
 finite number: a unit that is off adds nothing to any gradient, one that is on adds what
 its formula gives (dL/dz2 times its value).
 
-A bias of -inf gives the unit, for every pixel, what a bias of -1e30 gives: off.  Both
+A bias of -inf or NaN gives the unit, for every pixel, what a bias of -1e30 gives: off.  Both
 calls then do the same arithmetic, but for the order of the atomic sums over cells
 (300 of them at most, 300 x 2^-24 of the summed magnitudes): bar 1e-4 relative L2.
 """
@@ -46,13 +46,14 @@ def run(change):
     return float(loss.item()), out["sigma"].cpu().numpy(), {k: v.cpu().numpy().astype(np.float64) for k, v in dm.items()}
 
 
+@pytest.mark.parametrize("off", [-math.inf, math.nan])
 @pytest.mark.parametrize("units", [[5], [64, 65, 66, 67], [0, 9, 127]])
-def test_off_units(units):
+def test_off_units(units, off):
     def bias(x):
         def change(mlp, grid):
             mlp["b1"][units] = x
         return change
-    (l0, s0, g0), (l1, s1, g1) = run(bias(-math.inf)), run(bias(-1e30))
+    (l0, s0, g0), (l1, s1, g1) = run(bias(off)), run(bias(-1e30))
     assert np.array_equal(s0, s1) and l0 == pytest.approx(l1, rel=1e-5)
     assert not g0["w2"][units].any() and not g0["b1"][units].any() and not g0["w1"][units].any()
     for k in g0:
