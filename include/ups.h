@@ -48,7 +48,11 @@ typedef enum {
     UPS_ERR_ARG = 2,        /* invalid argument (sizes, NULL, alignment) */
     UPS_ERR_OOM = 3,        /* device or pinned allocation failed */
     UPS_ERR_CUDA = 4,       /* a CUDA runtime call failed */
-    UPS_ERR_TIMEOUT = 5,    /* a bounded wait ran out */
+    UPS_ERR_TIMEOUT = 5,    /* a bounded wait ran out.  One of a kernel's is told by the
+                               call that next waits for the GPU on its ups_ctx
+                               (ups_render_forward, ups_get_stats), or as the status of
+                               the requests of its batch; their results are not to be
+                               used. */
     UPS_ERR_CANCELLED = 6,  /* request cancelled before it ran */
     UPS_ERR_NONFINITE = 7,  /* check_finite found NaN/Inf in an input */
     UPS_ERR_CAPACITY = 8,   /* a fixed-size buffer is too small */

@@ -11,6 +11,7 @@
 
 #include "common.cuh"
 #include "decode_bwd.cuh"
+#include "lost_wait.cuh"
 #include "tiles.cuh"
 
 namespace ups {
@@ -143,16 +144,17 @@ struct ups_ctx {
     SortScratch sort;
     uint32_t *ikey_sorted = nullptr, *ival_sorted = nullptr;
     // device words of a forward and their pinned copy: the instance counters
-    // and the list flag (cleared by every forward), the error flag
+    // and the list flag (cleared by every forward)
     struct Words {
         unsigned long long n_inst[kInstCounters];
         int trunc_flag;  // set by the forward blend: a capped list was too short
-        int err;         // set by kernels whose bounded waits ran out
         uint32_t n_hits; // length of the last backward's hit list
     };
     Words *d_words = nullptr, *h_words = nullptr;
     cudaEvent_t words_ready = nullptr;  // the pinned copy has arrived
-    int *d_err = nullptr, *d_trunc_flag = nullptr;  // into d_words
+    int *d_trunc_flag = nullptr;         // into d_words
+    LostWait lost;                       // set by kernels whose bounded waits ran out
+    int *d_err = nullptr;                // its word on the device
     DevBuf trunc;                 // per-tile bit: the list cap cut the tile's list
     bool capped = false;          // the last forward capped its tile lists
     bool rowwise = false;         // the last forward built its lists row by row (bin.cu)
@@ -366,6 +368,9 @@ ups_status loss_views(ups_ctx *c, const ups_images *img, const ups_targets *tgt,
     stage_end(c, st, 1);
     return UPS_OK;
 }
+// The context's lost-wait word, for whoever ends the work of a stream.
+LostWait lost_wait(const ups_ctx *c) { return c->lost; }
+
 // Entries in the tile lists of the last forward (a capped forward keeps
 // fewer than there are instances unless the GPU rebuilt them whole: *refilled).
 // Synchronises the ctx stream.
@@ -458,6 +463,9 @@ ups_status ups_create(const ups_config *cfg, int device, ups_ctx **out) {
     e = cudaSetDevice(device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e == cudaSuccess) e = cudaMallocHost(&ctx->h_words, sizeof(ups_ctx::Words));
+    if (e == cudaSuccess) e = cudaHostAlloc(&ctx->lost.word, sizeof(int), cudaHostAllocMapped);
+    if (e == cudaSuccess) *ctx->lost.word = 0;
+    if (e == cudaSuccess) e = cudaHostGetDevicePointer(&ctx->d_err, ctx->lost.word, 0);
     if (e == cudaSuccess) e = cudaMalloc(&ctx->d_words, sizeof(ups_ctx::Words));
     if (e == cudaSuccess) e = cudaMemset(ctx->d_words, 0, sizeof(ups_ctx::Words));
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->words_ready, cudaEventDisableTiming);
@@ -466,7 +474,6 @@ ups_status ups_create(const ups_config *cfg, int device, ups_ctx **out) {
         ups_destroy(ctx);
         return UPS_ERR_CUDA;
     }
-    ctx->d_err = &ctx->d_words->err;
     ctx->d_trunc_flag = &ctx->d_words->trunc_flag;
     ctx->bp = BlendParams{c.alpha_min, c.alpha_max, c.t_min, c.dilation, c.near_z};
     *out = ctx;
@@ -481,6 +488,7 @@ ups_status ups_destroy(ups_ctx *c) {
                       &c->ival0, &c->ival1, &c->ranges, &c->g2, &c->hit_bits, &c->hit_list, &c->dec_scratch, &c->sort.hist, &c->trunc, &c->lift_scr, &c->ssim_g, &c->unc_scr, &c->anchor_scr};
     for (DevBuf *b : bufs) b->release();
     if (c->h_words) cudaFreeHost(c->h_words);
+    if (c->lost.word) cudaFreeHost(c->lost.word);
     if (c->h_anchor) cudaFreeHost(c->h_anchor);
     if (c->d_words) cudaFree(c->d_words);
     if (c->words_ready) cudaEventDestroy(c->words_ready);
@@ -610,7 +618,7 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     }
     uint4 *span = rowwise ? c->span.as<uint4>() : nullptr, *more = rowwise ? c->more.as<uint4>() : nullptr;
 
-    UPS_CUDA(c, cudaMemsetAsync(c->d_words, 0, offsetof(ups_ctx::Words, err), st));
+    UPS_CUDA(c, cudaMemsetAsync(c->d_words, 0, offsetof(ups_ctx::Words, n_hits), st));
     stage_begin(c, "project", st);
     if (k32)
         UPS_CUDA(c, launch_project_k32(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
@@ -644,9 +652,11 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
         stage_end(c, st, 2);
     }
     UPS_CUDA(c, cudaEventSynchronize(c->words_ready));
-    if (c->h_words->err != 0) {
-        cudaMemsetAsync(c->d_err, 0, sizeof(int), st);
-        return fail(c, UPS_ERR_TIMEOUT, "a bounded wait of a kernel ran out of polls in an earlier launch");
+    if (c->lost.take()) {
+        // (this call's own sort may be running: what it leaves belongs to this failure too)
+        cudaStreamSynchronize(st);
+        c->lost.take();
+        return fail(c, UPS_ERR_TIMEOUT, "a bounded wait of a kernel ran out of polls in this call or an earlier one");
     }
     uint64_t n_inst = 0;
     for (int i = 0; i < kInstCounters; ++i) n_inst += c->h_words->n_inst[i];
@@ -1065,6 +1075,9 @@ ups_status ups_get_stats(ups_ctx *c, ups_stats *out) {
     long long vis = 0;
     for (uint32_t x : h) vis += x > 0;
     out->n_visible = vis;
+    // the stream has ended: a wait that was lost is told here, not by the next forward
+    if (c->total_gv && c->lost.take())
+        return fail(c, UPS_ERR_TIMEOUT, "a bounded wait of a kernel ran out of polls: the last results are not to be used");
     return UPS_OK;
 }
 

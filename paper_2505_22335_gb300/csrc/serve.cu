@@ -19,6 +19,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "lost_wait.cuh"
 
 namespace ups {
 ups_status loss_views(ups_ctx *c, const ups_images *img, const ups_targets *tgt,
@@ -26,6 +27,7 @@ ups_status loss_views(ups_ctx *c, const ups_images *img, const ups_targets *tgt,
                       cudaStream_t st);
 ups_status render_forward_sets(ups_ctx *c, const ups_gaussians *g, const ups_camera *cams, int n_views,
                                const int *set_of_view, ups_images *out, ups_stream stream);
+LostWait lost_wait(const ups_ctx *c);
 }
 
 using namespace ups;
@@ -116,6 +118,7 @@ struct BatchDone {
     ups_server *srv;
     std::vector<Req *> reqs;
     size_t bytes;
+    LostWait lost;  // of the slot's context
 };
 
 void CUDART_CB on_batch_done(void *p) {
@@ -124,10 +127,14 @@ void CUDART_CB on_batch_done(void *p) {
     {
         std::lock_guard<std::mutex> lk(s->mu);
         const double t = s->now_ms();
+        // taken where the batch's kernels have ended and the slot's next ones have not
+        // begun, so that the loss is this batch's
+        const bool lost = bd->lost.take();
         for (Req *r : bd->reqs) {
             r->t_end = t;
-            if (r->status == UPS_PENDING) r->status = UPS_OK;
+            r->status = settled_status(r->status, lost);
         }
+        if (lost) s->err = "a bounded wait of a kernel ran out of polls";
         s->reserved -= bd->bytes;
         s->in_flight--;
     }
@@ -304,7 +311,7 @@ void worker(ups_server *s, int si) {
         std::string msg;
         ups_status st = run_batch(s, sl, batch, msg);
         if (st == UPS_OK) {
-            BatchDone *bd = new BatchDone{s, batch, bytes};
+            BatchDone *bd = new BatchDone{s, batch, bytes, lost_wait(sl.ctx)};
             if (cudaLaunchHostFunc(sl.st, on_batch_done, bd) != cudaSuccess) {
                 delete bd;
                 cudaStreamSynchronize(sl.st);
