@@ -552,7 +552,9 @@ ups_status ups_submit(ups_server *srv, const ups_request *req, uint64_t *ticket)
  * ticket. */
 ups_status ups_poll(ups_server *srv, uint64_t ticket, ups_result *out);
 /* As ups_poll, but blocks until the request is done, at most timeout_ms
- * (UPS_PENDING then). */
+ * (UPS_PENDING then; none or a negative one does not block, NaN is
+ * UPS_ERR_ARG).  Here and below a timeout of more than a year, infinity
+ * included, is a year. */
 ups_status ups_wait(ups_server *srv, uint64_t ticket, double timeout_ms, ups_result *out);
 /* Removes a request that has not started: UPS_OK (its poll then reports
  * UPS_ERR_CANCELLED), UPS_ERR_STATE if it already started. */

@@ -10,6 +10,7 @@
 // batch's memory reservation, which admits the next batch.
 #include <algorithm>
 #include <chrono>
+#include <cmath>
 #include <condition_variable>
 #include <deque>
 #include <mutex>
@@ -20,6 +21,7 @@
 
 #include "common.cuh"
 #include "lost_wait.cuh"
+#include "wait_span.cuh"
 
 namespace ups {
 ups_status loss_views(ups_ctx *c, const ups_images *img, const ups_targets *tgt,
@@ -478,10 +480,10 @@ ups_status ups_poll(ups_server *s, uint64_t ticket, ups_result *out) {
 // Woken by the end of a batch: a caller that polled every half millisecond saw a
 // tracking request of 3 ms a quarter of a millisecond late on average.
 ups_status ups_wait(ups_server *s, uint64_t ticket, double timeout_ms, ups_result *out) {
-    if (!s) return UPS_ERR_ARG;
+    if (!s || std::isnan(timeout_ms)) return UPS_ERR_ARG;
     std::unique_lock<std::mutex> lk(s->mu);
     s->waiters++;
-    s->cv.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms), [&] {
+    s->cv.wait_for(lk, wait_span(timeout_ms), [&] {
         auto it = s->reqs.find(ticket);
         return it == s->reqs.end() || it->second->status != UPS_PENDING;
     });
@@ -508,7 +510,7 @@ ups_status ups_cancel(ups_server *s, uint64_t ticket) {
 ups_status ups_server_wait_idle(ups_server *s, double timeout_ms) {
     if (!s) return UPS_ERR_ARG;
     std::unique_lock<std::mutex> lk(s->mu);
-    bool ok = s->cv.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms),
+    bool ok = s->cv.wait_for(lk, wait_span(timeout_ms),
                              [&] { return s->queue.empty() && s->in_flight == 0; });
     return ok ? UPS_OK : UPS_ERR_TIMEOUT;
 }
@@ -520,7 +522,7 @@ ups_status ups_server_set_scene(ups_server *s, const ups_anchors *scene, const u
     std::unique_lock<std::mutex> lk(s->mu);
     s->paused = true;
     // in_flight drops when a batch's stream work has completed (host callback)
-    const bool ok = s->cv.wait_for(lk, std::chrono::duration<double, std::milli>(timeout_ms),
+    const bool ok = s->cv.wait_for(lk, wait_span(timeout_ms),
                                    [&] { return s->in_flight == 0; });
     if (ok) {
         s->anc = *scene;
