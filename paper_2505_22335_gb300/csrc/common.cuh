@@ -26,7 +26,6 @@ struct DevView {
     float limx, limy;  // frustum guard on |X/Z|, |Y/Z|
     float t_norm;
     int set;        // the Gaussian set this view reads (attribute index set * n + g)
-    int set_first;  // 1: the first view reading that set
 };
 
 struct ViewTable {
@@ -121,7 +120,6 @@ struct DevBuf {
 struct SortScratch {
     DevBuf hist;
 };
-size_t radix_hist_bytes(size_t n);
 cudaError_t radix_sort_u32(uint32_t **key_io, uint32_t **key_alt, uint32_t **val_io,
                            uint32_t **val_alt, size_t n, int end_bit, SortScratch &s,
                            cudaStream_t st);

@@ -22,7 +22,7 @@ cudaError_t launch_project(const ViewTable &vt, const BlendParams &bp, int N, in
                            uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
 cudaError_t launch_project_k32(const ViewTable &vt, const BlendParams &bp, int N, int total, const ups_gaussians &g,
                                float4 *xyzo, float4 *conic, uint2 *rect, uint32_t *count, uint32_t *dkey32,
-                               uint32_t *dval, int vbits, uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
+                               int vbits, uint4 *span, uint4 *more, unsigned long long *n_inst, cudaStream_t st);
 cudaError_t launch_gather_counts(const uint32_t *sorted_gv, const uint32_t *count, uint32_t *out,
                                  int total, cudaStream_t st);
 cudaError_t launch_emit(const ViewTable &vt, const BlendParams &bp, int N, int total, const uint32_t *sorted_gv,
@@ -575,12 +575,8 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
         const int sv = !g->per_view ? 0 : set_of_view ? set_of_view[v] : v;
         if (sv < 0 || sv >= UPS_MAX_VIEWS) return fail(c, UPS_ERR_ARG, "set index out of range");
         vt.v[v].set = sv;
-        vt.v[v].set_first = 1;
         for (int u = 0; u < v; ++u)
-            if (vt.v[u].set == sv) {
-                vt.v[v].set_first = 0;
-                c->shared_sets = true;
-            }
+            if (vt.v[u].set == sv) c->shared_sets = true;
         if (set_of_view) c->n_sets = std::max(c->n_sets, sv + 1);
     }
     const size_t total = (size_t)g->n * n_views;
@@ -622,7 +618,7 @@ extern "C++" ups_status ups::render_forward_sets(ups_ctx *c, const ups_gaussians
     stage_begin(c, "project", st);
     if (k32)
         UPS_CUDA(c, launch_project_k32(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),
-                                       c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint32_t>(), nullptr, vbits,
+                                       c->rect.as<uint2>(), c->count.as<uint32_t>(), c->dkey0.as<uint32_t>(), vbits,
                                        span, more, c->d_words->n_inst, st));
     else
         UPS_CUDA(c, launch_project(vt, c->bp, c->N, (int)total, *g, c->xyzo.as<float4>(), c->conic.as<float4>(),

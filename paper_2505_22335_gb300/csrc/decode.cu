@@ -4,8 +4,8 @@
 // Row = (anchor, view).  MLP input x = [f_v, delta_vc, d_vc, sin(pi t),
 // cos(pi t)]; four MLPs (opacity, covariance, colour: ReLU hidden; feature
 // F_d: SoftPlus hidden) of width `hidden` = 32.  Weights live in shared memory
-// and are read as float4 broadcasts (every lane of a warp reads the same
-// weight), so the inner loops are FMA-bound.
+// and are read as 16-byte broadcasts (every lane of a warp reads the same
+// weight); what bounds the loops stands at each kernel.
 //
 // Backward (FP32 data path): one thread per row recomputes each MLP group's
 // hidden layer, forms dL/dY of the group's outputs and propagates it to the
@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(dbwd::kRowsFp32, dbwd::kRowsCtasPerSm) k_decod
     const int n_out = dbwd::n_out(a.K, NF);
     const DecodeArgs da{a.A, a.K, NF, n_out, a.pos, a.afeat, a.offs, a.ascale, a.w1, a.b1, a.w2, a.b2, a.op_tanh};
     // W1 transposed [38][128] (inputs x hidden), b1, W2 [n_out][32], b2, and
-    // the per-row input gradients dx [36][128 rows]
+    // the per-row input gradients dx [36][256 rows]
     float *sW1T = sm, *sb1 = sW1T + kDin * 4 * kH, *sW2 = sb1 + 4 * kH, *sb2 = sW2 + n_out * kH;
     float *sDXall = sb2 + ((n_out + 3) & ~3);
     load_weights_T(da, sW1T, sb1, sW2, sb2);
@@ -656,8 +656,6 @@ size_t fwd_smem(int n_out, int warps) {
 }
 
 }  // namespace
-
-size_t decode_bwd_rows_fp32_smem(int K, int NF) { return bwd_rows_smem(dbwd::n_out(K, NF)); }
 
 cudaError_t launch_live_rows(const dbwd::Args &a, int V, uint32_t *rows, uint32_t *n_rows, cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(n_rows, 0, sizeof(uint32_t), st);

@@ -11,8 +11,10 @@
 // A product whose tiles are too few to fill the GPU is split along K over
 // grid.z, the parts added with atomics into C after C was scaled by beta.  With
 // parts of at most 256 asked for, a product with enough tiles adds the same
-// parts in order in one CTA: its elements then do not depend on how many rows
-// are multiplied at once.  The next operand tiles are loaded while the current
+// parts in order in one CTA: up to two parts (K <= 512) its elements then do not
+// depend on how many rows are multiplied at once; of more, the split product's
+// atomics add in any order, and elements differ in their last bits from run to
+// run.  The next operand tiles are loaded while the current
 // ones are multiplied.
 #include <algorithm>
 

@@ -183,7 +183,6 @@ extern "C" ups_status ups_render_forward_static(const ups_config *cfg, const ups
     const int N = g->n, per_view = g->per_view ? 1 : 0;
     for (int v = 0; v < n_views; ++v) {
         vt.v[v].set = per_view ? v : 0;
-        vt.v[v].set_first = per_view || v == 0;
     }
 
     unsigned char *base = nullptr;

@@ -345,7 +345,9 @@ cudaError_t radix_fixed(K **key_io, K **key_alt, uint32_t **val_io, uint32_t **v
 // input (a ticket, so that every earlier tile is already running or done),
 // ranks its items by ballots, publishes its 256 digit counts and finds the
 // items before it by walking back over the earlier tiles' published counts until
-// one holds its inclusive sum.  Every wait on a published count is bounded: a
+// one holds its inclusive sum (the "decoupled look-back" of Merrill and Garland's
+// single-pass prefix scan, 2016, applied to digit counts as in Adinets and Merrill's
+// Onesweep, 2022).  Every wait on a published count is bounded: a
 // wait that runs out sets *err and ends the CTA (its consumers take no id on trust:
 // list_rules.cuh, k_gather_counts and k_emit).  The first pass makes up the values (the positions) and the last
 // one writes no keys.  Held by the ranking's ballots and the walk back, not by
@@ -656,12 +658,6 @@ cudaError_t radix_sort_u64_fixed(uint64_t **key_io, uint64_t **key_alt, uint32_t
 size_t scan_scratch_bytes(size_t n) {
     size_t nb = (n + kScanTile - 1) / kScanTile + 1;
     return 256 + nb * sizeof(uint64_t);
-}
-
-size_t radix_hist_bytes(size_t n) {
-    size_t nblocks = (n + Radix<uint64_t>::tile - 1) / Radix<uint64_t>::tile;
-    size_t hist_n = (size_t)kBins * nblocks;
-    return hist_n * 4 + 256 + scan_scratch_bytes(hist_n);
 }
 
 cudaError_t radix_sort_u32(uint32_t **key_io, uint32_t **key_alt, uint32_t **val_io,

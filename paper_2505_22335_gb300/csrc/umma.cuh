@@ -75,15 +75,6 @@ __device__ __forceinline__ void mma(uint32_t tmem_d, uint64_t a, uint64_t b, uin
                      "l"(a), "l"(b), "r"(id), "r"(acc));
 }
 
-// kind::f16 MMA with A in tensor memory (rows in lanes, K along columns, two
-// 16-bit elements per 32-bit column, the lower K index in the low half) and B
-// from a shared-memory descriptor
-__device__ __forceinline__ void mma_f16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t id, uint32_t acc) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(tmem_d),
-                 "r"(tmem_a), "l"(b), "r"(id), "r"(acc));
-}
-
 __device__ __forceinline__ void commit(uint64_t *mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
         smem_addr(mbar)));
@@ -103,6 +94,9 @@ __device__ __forceinline__ void mma_warp(uint32_t tmem_d, uint64_t a, uint64_t b
                      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
                      "l"(a), "l"(b), "r"(id), "r"(acc));
 }
+// kind::f16 MMA with A in tensor memory (rows in lanes, K along columns, two
+// 16-bit elements per 32-bit column, the lower K index in the low half) and B
+// from a shared-memory descriptor
 __device__ __forceinline__ void mma_f16_ts_warp(uint32_t tmem_d, uint32_t tmem_a, uint64_t b, uint32_t id,
                                                 uint32_t acc) {
     asm volatile("{\n.reg .pred p, e;\nsetp.ne.b32 p, %4, 0;\nelect.sync _|e, 0xffffffff;\n"
@@ -130,16 +124,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *mbar, uint32_t parity, int l
                      : "=r"(done)
                      : "r"(smem_addr(mbar)), "r"(parity));
     return done != 0;
-}
-
-// bulk copy (TMA, untiled) global -> shared, completing `bytes` of the
-// transaction count of *mbar; both addresses 16-byte aligned, bytes a multiple
-// of 16
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                     smem_addr(dst)),
-                 "l"(src), "r"(bytes), "r"(smem_addr(mbar))
-                 : "memory");
 }
 
 // arrive on *mbar (one of its expected arrivals) and add `bytes` to the
