@@ -317,10 +317,12 @@ void worker(ups_server *s, int si) {
             if (cudaLaunchHostFunc(sl.st, on_batch_done, bd) != cudaSuccess) {
                 delete bd;
                 cudaStreamSynchronize(sl.st);
+                lost_wait(sl.ctx).take();
                 finish_now(s, batch, bytes, UPS_ERR_CUDA);
             }
         } else {
             cudaStreamSynchronize(sl.st);
+            lost_wait(sl.ctx).take();  // of this batch, which fails as it is
             {
                 std::lock_guard<std::mutex> lk(s->mu);
                 s->err = msg;
