@@ -234,14 +234,14 @@ ALU_STAGES = {"decode_fwd", "decode_bwd_rows", "composite_fwd", "composite_bwd"}
 # the kernel's source file when it was captured).  Reported as the roofline's `traffic` only while
 # the source file still has that hash; any later change of the kernel makes it null (stale).
 MEASURED_TRAFFIC = {
-    # full ncu captures of one launch on the 2-view profiling workload (1M Gaussians, 2 x 640x480), scaled to the
+    # ncu captures (DRAM bytes) of one launch on the 2-view profiling workload (1M Gaussians, 2 x 640x480), scaled to the
     # 8-view launch by the list entries the tiles read (384,532 -> 1,618,003; images scale alike, 4x the pixels)
-    ("composite_bwd", DEFAULT_WORKLOAD): (301.7e6, "2026-12-04 (2-view capture x 4.21)", "cb96ae212ea91e15"),
-    ("composite_fwd", DEFAULT_WORKLOAD): (107.4e6, "2026-12-04 (2-view capture x 4.21)", "cb96ae212ea91e15"),
-    # full ncu capture of one 200,000-row launch on the 2-view profiling workload; the 8-view step's 4 launches
+    ("composite_bwd", DEFAULT_WORKLOAD): (300.7e6, "2026-12-05 (2-view capture x 4.21)", "ab97c90f1b2c903b"),
+    ("composite_fwd", DEFAULT_WORKLOAD): (97.7e6, "2026-12-05 (2-view capture x 4.21)", "ab97c90f1b2c903b"),
+    # ncu capture of one 200,000-row launch on the 2-view profiling workload; the 8-view step's 4 launches
     # average the same 200,000 rows, and the traffic is per row (dL/dG read, scratch written)
-    ("decode_bwd_rows", DEFAULT_WORKLOAD): (786.9e6, "2026-12-04 (2-view capture, 200k rows = the average launch)",
-                                            "ef771be9ad95a383"),
+    ("decode_bwd_rows", DEFAULT_WORKLOAD): (785.7e6, "2026-12-05 (2-view capture, 200k rows = the average launch)",
+                                            "19e525e4aef1d3e5"),
 }
 STAGE_SOURCE = {"composite_fwd": "composite.cu", "composite_bwd": "composite.cu", "decode_bwd_rows": "decode.cu",
                 "decode_fwd": "decode.cu", "decode_wgrad": "wgrad_tc.cu", "project_bwd": "project.cu"}
